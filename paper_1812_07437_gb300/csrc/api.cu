@@ -242,7 +242,10 @@ static void free_all(cov_handle* h) {
                   h->Srows, h->cosmo_d, h->Fsig,  h->Esig,    h->Msig,   h->FsigT,  h->EsigT,     h->MsigT,
                   h->invN,  h->omN,   h->work,    h->chol_scratch, h->chol_status, h->mb, h->omb, h->cs,
                   h->cw,    h->sigF,  h->ac,      h->bmask,   h->gblk,   h->wait_flag, h->pca_buf,
-                  h->kap,   h->kgram, h->kcol,    h->kn,      h->koff,      h->plist};
+                  h->kap,   h->kgram, h->kcol,    h->kn,      h->koff,      h->plist,
+                  h->knode, h->kwt,   h->kw8,     h->kws,     h->zsrc,      h->gsel,    h->cmass,   h->chebm,
+                  h->trigeo, h->zint, h->pk,      h->amp_part, h->Draw,     h->chis,    h->cz,      h->rvir,
+                  h->hint,  h->qw,    h->proj,    h->ksum,    h->kticket};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (h->tile_ring) cudaFree(h->tile_ring);
@@ -290,6 +293,21 @@ static void init_allocs(cov_handle* h, std::vector<std::pair<void**, size_t>>& a
       {(void**)&h->B1h3, d * ntri * nchi},  {(void**)&h->Ps, d * nl * nt * nt},
       {(void**)&h->B1hp, d * ntri * nt * nt * nt},
       {(void**)&h->cosmo_d, sizeof(cov_cosmology)},
+      {(void**)&h->knode, d * WL_N_K},      {(void**)&h->kwt, d * WL_N_K},
+      {(void**)&h->kw8, d * WL_N_K},        {(void**)&h->kws, d * WL_N_K},
+      {(void**)&h->pk, d * WL_N_K},         {(void**)&h->amp_part, d * (WL_N_K / WL_KT_THREADS)},
+      {(void**)&h->zsrc, d * nt * WL_N_ZS}, {(void**)&h->gsel, d * nt * WL_N_ZS * nt},
+      {(void**)&h->chis, d * nt * WL_N_ZS}, {(void**)&h->chebm, d * WL_N_CH * WL_N_CH},
+      {(void**)&h->zint, d * WL_N_ZI * WL_ZI_STRIDE},
+      {(void**)&h->cmass, d * nmb},         {(void**)&h->rvir, d * nmb},
+      {(void**)&h->ksum, d * 3 * WL_KSPLIT * (nchi + nmb)},
+      {(void**)&h->kticket, 4 * (nchi + nmb)},
+      {(void**)&h->Draw, d * nchi},         {(void**)&h->cz, d * nchi},
+      {(void**)&h->trigeo, d * WL_TRI_GEO * ntri},
+      // halo integrals: I_2^0, I_1^1, I_1^2 per ell bin, I_2^1, I_2^2 per bin pair, I_3^0, I_3^1 per triple
+      {(void**)&h->hint, d * (3 * nl + nl * (nl + 1) + 2 * ntri) * nchi},
+      {(void**)&h->qw, d * (nt * (nt + 1) / 2 + nt * (nt + 1) * (nt + 2) / 6) * nchi},
+      {(void**)&h->proj, d * (nl * (nt * (nt + 1) / 2) + ntri * (nt * (nt + 1) * (nt + 2) / 6))},
   };
 }
 
@@ -398,6 +416,7 @@ extern "C" int cov_init(const cov_cosmology* cosmo, const cov_nz* nz, const cov_
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(h->rowdesc_d, h->rowdesc.data(), 4 * h->rowdesc.size(), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->scal, 0, d * SC_N, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(h->kticket, 0, 4 * (size_t)(h->nchi + h->nmb), s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(h->cosmo_d, &h->cosmo, sizeof(cov_cosmology), cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) {
     g_init_err = std::string("upload: ") + cudaGetErrorString(e);

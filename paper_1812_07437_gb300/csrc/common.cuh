@@ -38,9 +38,22 @@
 #define WL_LNK_MIN (-11.512925464970229)  // ln 1e-5
 #define WL_LNK_MAX (6.907755278982137)    // ln 1e3
 #define WL_FD_H 1.0e-3     // ln k step of the 4th-order differences
+#define WL_N_ZI 64         // intervals of the piecewise chi(z) on [0, z_max]
+#define WL_N_CH 12         // Chebyshev nodes of 1 / E(z) per interval
+#define WL_ZI_STRIDE 32    // doubles per interval: 13 of the integral, 12 of 1 / E, the whole integral
+#define WL_ZI_DER 13
+#define WL_ZI_TOT 25
+#define WL_KT_THREADS 64   // threads (and k nodes) per block of the linear-spectrum table
+#define WL_KSPLIT 4        // blocks that share one sum over the k nodes
+#define WL_TRI_GEO 42      // per triple: F2 of the three leg pairs, their cosines, F2 of the 12 shifted shapes
 
 // scalars kept on the device (index into h->scal)
 enum { SC_CHIMAX = 0, SC_AMP = 1, SC_NOISE = 2, SC_D1 = 3, SC_STATUS = 7, SC_N = 8 };
+
+// cosmology-only factors of the Eisenstein & Hu transfer function
+struct EhConst {
+  double ks, al, omh, th2;  // 0.43 h s, alpha_Gamma, Omega_m h, (T_cmb / 2.7)^2
+};
 
 struct DevCosmo {
   double Om, Ob, h, ns, sigma8, w0, Tcmb;
@@ -127,6 +140,20 @@ struct cov_handle {
   double *f = nullptr, *b1 = nullptr, *b2 = nullptr, *U = nullptr, *Pl = nullptr, *dPl = nullptr;
   double* Psh = nullptr;  // [n_ell][n_chi][4] P_lin at the shifted k of the ln k differences
   double *zedges = nullptr, *norms = nullptr, *W = nullptr, *sigw2 = nullptr;
+  // binning- and n(z)-only tables of the builders, made once (wl_quadrature):
+  // the sigma rule's k nodes and weights, the source nodes of the fixed pieces
+  // between tomographic edges with their n(z) P_i weights, the Duffy mass
+  // factors, the Chebyshev matrix of the chi(z) intervals and the triangles' shapes
+  double *knode = nullptr, *kwt = nullptr, *kw8 = nullptr, *kws = nullptr;
+  double *zsrc = nullptr, *gsel = nullptr, *cmass = nullptr, *chebm = nullptr, *trigeo = nullptr;
+  // rebuilt for every cosmology: chi intervals, k^ns T^2 on the k nodes with
+  // the partial sigma_8 sums, growth before normalisation, chi and 1 / chi at the
+  // source nodes, (1 + z)^C and r_vir, halo integrals [item][n_chi], Limber weights,
+  // projected spectra per symmetric tomographic multiset
+  double *zint = nullptr, *pk = nullptr, *amp_part = nullptr, *Draw = nullptr, *chis = nullptr, *cz = nullptr;
+  double* ksum = nullptr;   // [sum][WL_KSPLIT][3] parts of the sums over the k nodes
+  int* kticket = nullptr;   // [sum] parts delivered so far (zero between launches)
+  double *rvir = nullptr, *hint = nullptr, *qw = nullptr, *proj = nullptr;
   int64_t *slo_d = nullptr, *shi_d = nullptr, *Nmodes = nullptr, *Ntri = nullptr;
   int32_t* rowtab = nullptr;  // [nl][2][rmax+1]: x_outer, x_inner per row
   int32_t *tris_d = nullptr, *rowdesc_d = nullptr;
@@ -243,6 +270,7 @@ void wl_stage_end(cov_handle* h, int token, cudaStream_t s);
 // ---- stage entry points (one per translation unit) -------------------------
 int wl_quadrature(cov_handle* h, cudaStream_t s);  // tables.cu
 int wl_tables(cov_handle* h, cudaStream_t s);   // tables.cu
+int wl_triangle_shapes(cov_handle* h, cudaStream_t s);  // spectra.cu: once per handle
 int wl_counts(cov_handle* h, cudaStream_t s);   // counts.cu
 int wl_couplings(cov_handle* h, cudaStream_t s);  // coupling.cu: exact BB+PT couplings (synchronises s)
 void wl_coupling_plan(cov_handle* h);             // coupling.cu: columns per bin (host)
@@ -282,142 +310,178 @@ __device__ __forceinline__ DevCosmo dev_cosmo(const cov_cosmology& c) {
   return DevCosmo{c.Om, c.Ob, c.h, c.ns, c.sigma8, c.w0, c.Tcmb};
 }
 
-// E(z) = H(z)/H0 for flat w0-CDM
-__device__ __forceinline__ double dev_E(double z, const cov_cosmology& c) {
-  double zp1 = 1.0 + z;
-  return sqrt(c.Om * zp1 * zp1 * zp1 + (1.0 - c.Om) * pow(zp1, 3.0 * (1.0 + c.w0)));
+// d(chi H0 / c) / dy at y = ln(1 + z) for flat w0-CDM: e^y / E, E = H / H0
+__device__ __forceinline__ double dev_dchi_dy(double y, const cov_cosmology& c) {
+  const double a1 = exp(y);
+  return a1 * rsqrt(c.Om * a1 * a1 * a1 + (1.0 - c.Om) * exp(3.0 * (1.0 + c.w0) * y));
 }
 
-// chi(z) with the 64-node Gauss-Legendre rule on [0, z]
-__device__ __forceinline__ double dev_chi_of_z(double z, const cov_cosmology& c, const double* glx,
-                                               const double* glw) {
-  double s = 0.0;
-  for (int i = 0; i < WL_N_GL_CHI; ++i) {
-    double zz = 0.5 * z * (glx[i] + 1.0);
-    s += glw[i] / dev_E(zz, c);
+// ---- chi(z) as a piecewise polynomial in y = ln(1 + z) ------------------------
+// chi H0 / c = int e^y / E dy.  [0, ln(1 + z_max)] is cut into WL_N_ZI equal
+// intervals, each holding the integrated Chebyshev interpolant of the integrand
+// (WL_N_CH nodes).  The integrand's singularities lie at |Im y| ~ 1, so the
+// interpolant is good to rounding (its coefficients fall by ~1/190 each at
+// z_max = 3, by ~1/39 at z_max = 1000), and one evaluation costs ~25 operations
+// where the direct 64-node rule on [0, z] costs 64 evaluations of E.
+// sum_k b_k T_k(t), t in [-1, 1], by Clenshaw
+__device__ __forceinline__ double dev_clenshaw(const double* b, int n, double t) {
+  double u1 = 0.0, u2 = 0.0;
+  const double t2 = 2.0 * t;
+  for (int k = n - 1; k >= 1; --k) {
+    const double u0 = fma(t2, u1, b[k] - u2);
+    u2 = u1;
+    u1 = u0;
   }
-  return WL_C_OVER_H0 * 0.5 * z * s;
+  return fma(t, u1, b[0] - u2);
+}
+// chi H0 / c at y; cum[j]: the integral up to interval j
+__device__ __forceinline__ double dev_chi_unit(double y, double ymax, const double* zint, const double* cum) {
+  const double s = y / ymax * WL_N_ZI;
+  int j = (int)s;
+  j = j < 0 ? 0 : (j > WL_N_ZI - 1 ? WL_N_ZI - 1 : j);
+  return cum[j] + dev_clenshaw(zint + j * WL_ZI_STRIDE, WL_N_CH + 1, 2.0 * (s - j) - 1.0);
 }
 
 // Eisenstein & Hu (1998) no-wiggle transfer function, k in h/Mpc
-__device__ __forceinline__ double dev_eh_T(double k, const cov_cosmology& c) {
+__device__ __forceinline__ EhConst dev_eh_const(const cov_cosmology& c) {
   double omh2 = c.Om * c.h * c.h, obh2 = c.Ob * c.h * c.h, fb = c.Ob / c.Om;
   double th = c.Tcmb / 2.7;
-  double s = 44.5 * log(9.83 / omh2) / sqrt(1.0 + 10.0 * pow(obh2, 0.75));
+  double s = 44.5 * log(9.83 / omh2) / sqrt(1.0 + 10.0 * sqrt(obh2 * sqrt(obh2)));
   double al = 1.0 - 0.328 * log(431.0 * omh2) * fb + 0.38 * log(22.3 * omh2) * fb * fb;
-  double ks = 0.43 * k * c.h * s;
+  return EhConst{0.43 * c.h * s, al, c.Om * c.h, th * th};
+}
+
+__device__ __forceinline__ double dev_eh_T(double k, const EhConst& e) {
+  double ks = k * e.ks;
   double ks2 = ks * ks;
-  double geff = c.Om * c.h * (al + (1.0 - al) / (1.0 + ks2 * ks2));
-  double q = k * th * th / geff;
+  double geff = e.omh * (e.al + (1.0 - e.al) / (1.0 + ks2 * ks2));
+  double q = k * e.th2 / geff;
   double L0 = log(2.0 * 2.718281828459045 + 1.8 * q);
   double C0 = 14.2 + 731.0 / (1.0 + 62.5 * q);
   return L0 / (L0 + C0 * q * q);
 }
 
-__device__ __forceinline__ double dev_plin(double k, double Dg, double amp, const cov_cosmology& c) {
-  double T = dev_eh_T(k, c);
-  return amp * pow(k, c.ns) * T * T * Dg * Dg;
+// k^ns T(k)^2: P_lin = amplitude x this x D^2
+__device__ __forceinline__ double dev_plin_unit(double k, const EhConst& e, double ns) {
+  double T = dev_eh_T(k, e);
+  return pow(k, ns) * T * T;
 }
 
-__device__ __forceinline__ double dev_dplin(double k, double Dg, double amp, const cov_cosmology& c) {
-  const double h = WL_FD_H;
-  double f2 = dev_plin(k * exp(2 * h), Dg, amp, c), f1 = dev_plin(k * exp(h), Dg, amp, c);
-  double m1 = dev_plin(k * exp(-h), Dg, amp, c), m2 = dev_plin(k * exp(-2 * h), Dg, amp, c);
-  return (-f2 + 8.0 * f1 - 8.0 * m1 + m2) / (12.0 * h);
-}
-
-// spherical top-hat window and its derivative (Taylor series below x = 0.5)
-__device__ __forceinline__ double dev_tophat(double x) {
+// spherical top-hat window W and its derivative dW (Taylor series below
+// x = 0.5); one sine, one cosine and one reciprocal serve both
+__device__ __forceinline__ void dev_tophat(double x, double* W, double* dW) {
   if (x < 0.5) {
-    // coefficients 3 (-1)^n (2n+2)/(2n+3)!, n = 0..6
-    const double c[7] = {1.0, -0.1, 1.0 / 280.0, -1.0 / 15120.0, 1.0 / 1330560.0, -1.0 / 172972800.0,
-                         1.0 / 31135104000.0};
-    double x2 = x * x, acc = 0.0;
-    for (int n = 6; n >= 0; --n) acc = acc * x2 + c[n];
-    return acc;
-  }
-  double sx, cx;
-  sincos(x, &sx, &cx);
-  return 3.0 * (sx - x * cx) / (x * x * x);
-}
-
-__device__ __forceinline__ double dev_dtophat(double x) {
-  if (x < 0.5) {
-    // 2n c_n for n = 1..7
-    const double c[8] = {0.0, -0.1, 1.0 / 280.0, -1.0 / 15120.0, 1.0 / 1330560.0, -1.0 / 172972800.0,
+    // coefficients 3 (-1)^n (2n+2)/(2n+3)!, n = 0..7; the derivative's are 2n times these
+    const double c[8] = {1.0, -0.1, 1.0 / 280.0, -1.0 / 15120.0, 1.0 / 1330560.0, -1.0 / 172972800.0,
                          1.0 / 31135104000.0, -1.0 / 7410154752000.0};
-    double x2 = x * x, acc = 0.0;
-    for (int n = 7; n >= 1; --n) acc = acc * x2 + 2.0 * n * c[n];
-    return acc * x;
-  }
-  double sx, cx;
-  sincos(x, &sx, &cx);
-  return 3.0 * ((x * x - 3.0) * sx + 3.0 * x * cx) / (x * x * x * x);
-}
-
-// Sine and cosine integrals Si(x), Ci(x) for x > 0.
-// x <= 4: the power series Si = sum (-1)^k x^(2k+1)/((2k+1)(2k+1)!),
-//         Ci = gamma + ln x + sum_{k>=1} (-1)^k x^(2k)/(2k (2k)!).
-// x > 4:  E1(ix) = -Ci(x) + i (Si(x) - pi/2) from the continued fraction
-//         E1(z) = e^-z / (z + 1 - 1^2/(z + 3 - 2^2/(z + 5 - ...))) evaluated by
-//         the modified Lentz method (Lentz 1976; Thompson & Barnett 1986).
-__device__ __forceinline__ void dev_sici(double x, double* si, double* ci) {
-  if (x <= 4.0) {
-    double x2 = x * x;
-    double ts = x, ssum = x;  // (-1)^k x^(2k+1)/(2k+1)!
-    double tc = 1.0, csum = 0.0;  // (-1)^k x^(2k)/(2k)!
-    for (int k = 1; k < 60; ++k) {
-      double tk = 2.0 * k;
-      tc *= -x2 / ((tk - 1.0) * tk);
-      csum += tc / tk;
-      ts *= -x2 / (tk * (tk + 1.0));
-      ssum += ts / (tk + 1.0);
-      if (fabs(ts) < 1e-18 * fabs(ssum) && fabs(tc) < 1e-18) break;
-    }
-    *si = ssum;
-    *ci = WL_EULER_GAMMA + log(x) + csum;
+    double x2 = x * x, acc = 0.0, dcc = 0.0;
+#pragma unroll
+    for (int n = 6; n >= 0; --n) acc = acc * x2 + c[n];
+#pragma unroll
+    for (int n = 7; n >= 1; --n) dcc = dcc * x2 + 2.0 * n * c[n];
+    *W = acc;
+    *dW = dcc * x;
     return;
   }
-  const double tiny = 1e-300;
-  // complex arithmetic on (re, im)
-  double br = 1.0, bi = x;              // b = 1 + i x
-  double cr = 1.0 / tiny, ci_ = 0.0;    // c
-  double den = br * br + bi * bi;
-  double dr = br / den, di = -bi / den; // d = 1/b
-  double hr = dr, hi = di;              // h = d
-  for (int i = 2; i < 400; ++i) {
-    double a = -(double)(i - 1) * (i - 1);
-    br += 2.0;
-    // d = 1/(a d + b)
-    double tr = a * dr + br, ti = a * di + bi;
-    den = tr * tr + ti * ti;
-    dr = tr / den;
-    di = -ti / den;
-    // c = b + a/c
-    den = cr * cr + ci_ * ci_;
-    double acr = a * cr / den, aci = -a * ci_ / den;
-    cr = br + acr;
-    ci_ = bi + aci;
-    // del = c d ; h *= del
-    double er = cr * dr - ci_ * di, ei = cr * di + ci_ * dr;
-    double nr = hr * er - hi * ei, ni = hr * ei + hi * er;
-    hr = nr;
-    hi = ni;
-    if (fabs(er - 1.0) + fabs(ei) < 1e-16) break;
-  }
   double sx, cx;
   sincos(x, &sx, &cx);
-  // E1(ix) = (cos x - i sin x) h
-  double er = cx * hr + sx * hi, ei = cx * hi - sx * hr;
-  *ci = -er;
-  *si = 0.5 * WL_PI + ei;
+  double iv = 1.0 / x, iv3 = 3.0 * (iv * iv) * iv;
+  *W = (sx - x * cx) * iv3;
+  *dW = ((x * x - 3.0) * sx + 3.0 * x * cx) * (iv3 * iv);
 }
 
-// Normalised truncated-NFW Fourier profile u(k|m) with the mean-density
-// (200 x rho_com) mass definition and the Duffy et al. (2008) concentration.
-// median concentration c(m, z) (Duffy et al. 2008, 200 x mean density)
-__device__ __forceinline__ double dev_conc(double m, double z) {
-  return WL_DUFFY_A * pow(m / WL_DUFFY_MPIVOT, WL_DUFFY_B) * pow(1.0 + z, WL_DUFFY_C);
+// Auxiliary functions of the sine and cosine integrals (Abramowitz & Stegun
+// 5.2.6-5.2.7): f(x) = Ci(x) sin x + (pi/2 - Si(x)) cos x,
+// g(x) = -Ci(x) cos x + (pi/2 - Si(x)) sin x, for x >= 4.  x f and x^2 g are
+// Stieltjes functions of 1/x^2, so rational forms in 1/x^2 converge fast and
+// have positive coefficients only (no cancellation): least-squares fits on
+// Chebyshev nodes of (0, 1/16] in 50-digit arithmetic, relative error below
+// 2e-17 (f, degree 10) and 8e-18 (g, degree 11).
+__device__ __forceinline__ void dev_sici_fg(double x, double ix, double* f, double* g) {
+  const double fn[11] = {0.99999999999999998378, 928.05420382076693203, 311792.70383167412804,
+                         49241850.478246443474,  3978741250.1625408183, 167994398922.03792598,
+                         3636504135501.9774993,  37980955670999.667919, 168886251080155.99331,
+                         244439194595624.65367,  50540378205319.638131};
+  const double fd[11] = {1.0,
+                         930.05420382076576918,
+                         313628.81223932914864,
+                         49847506.801771428012,
+                         4071538491.4537409714,
+                         175133077250.8030367,
+                         3915194333202.1978355,
+                         43309300071250.424812,
+                         214523982278849.61302,
+                         390009839291757.9415,
+                         160657256290782.04942};
+  const double gn[12] = {0.99999999999999999237, 1275.0091795677156003, 605421.35439380592647,
+                         139649577.9133789602,   17136978224.50301275,  1153313898494.0901147,
+                         42382981825994.469923,  821420612961746.69728, 7801194798999991.8498,
+                         31529642294798734.145,  39893722197823414.851, 4895049205879604.8997};
+  const double gd[12] = {1.0,
+                         1281.0091795677148263,
+                         612987.40947122489641,
+                         143178821.26857615156,
+                         17928586069.529463862,
+                         1246368476448.8059744,
+                         48253850554104.998422,
+                         1017580800246133.922,
+                         11111072139559062.084,
+                         57203395181087421.55,
+                         116198203079107446.44,
+                         61464150475231224.378};
+  const double s = ix * ix;
+  double a = fn[10], b = fd[10], c = gn[11], d = gd[11];
+#pragma unroll
+  for (int i = 9; i >= 0; --i) {
+    a = fma(a, s, fn[i]);
+    b = fma(b, s, fd[i]);
+  }
+#pragma unroll
+  for (int i = 10; i >= 0; --i) {
+    c = fma(c, s, gn[i]);
+    d = fma(d, s, gd[i]);
+  }
+  const double r = 1.0 / (b * d);
+  *f = ix * a * (d * r);
+  *g = s * c * (b * r);
+}
+
+// Si(x) / x and (Ci(x) - gamma - ln x) / x^2 for 0 < x <= 4: entire functions
+// of x^2, Chebyshev interpolants of degree 11 (errors below 1e-19) written as
+// polynomials.
+__device__ __forceinline__ void dev_sici_small(double x2, double* p, double* q) {
+  const double P[12] = {1.0,
+                        -0.055555555555555554183,
+                        0.0016666666666666625773,
+                        -0.000028344671201809284662,
+                        3.0619243581918498966e-7,
+                        -2.2774643976507699453e-9,
+                        1.2353110412022082067e-11,
+                        -5.0981057067843259861e-14,
+                        1.6537641118389194423e-16,
+                        -4.3243943635141795944e-19,
+                        9.2258372308936945248e-22,
+                        -1.4510986112315725863e-24};
+  const double Q[12] = {-0.25,
+                        0.010416666666666666615,
+                        -0.00023148148148148132892,
+                        3.1001984126982345943e-6,
+                        -2.7557319223878443742e-8,
+                        1.739729748606424921e-10,
+                        -8.1933896262629766677e-13,
+                        2.9871720472757203718e-15,
+                        -8.6772094614299662671e-18,
+                        2.0543184505162214002e-20,
+                        -4.0087791977665931461e-23,
+                        5.8582225667303094627e-26};
+  double a = P[11], b = Q[11];
+#pragma unroll
+  for (int i = 10; i >= 0; --i) {
+    a = fma(a, x2, P[i]);
+    b = fma(b, x2, Q[i]);
+  }
+  *p = a;
+  *q = b;
 }
 
 // u(k | m, c) for c < 1 from its defining integral in t = r / r_vir:
@@ -441,20 +505,43 @@ __device__ __forceinline__ double dev_nfw_u_integral(double K, double c, const d
   return num / den;
 }
 
-// normalised Fourier transform u(k | m, c) of the truncated NFW profile: the
-// closed form in sine/cosine integrals for c >= 1, the defining integral below
-__device__ __forceinline__ double dev_nfw_u(double k, double m, double c, double rho, const double* x16,
-                                           const double* w16) {
-  double rv = cbrt(3.0 * m / (4.0 * WL_PI * WL_DELTA_VIR * rho));
-  if (c < WL_NFW_C_INTEGRAL) return dev_nfw_u_integral(k * rv, c, x16, w16);
-  double x = k * rv / c;
-  double s1, c1, s2, c2;
-  dev_sici(x, &s1, &c1);
-  dev_sici((1.0 + c) * x, &s2, &c2);
-  double sx, cx;
-  sincos(x, &sx, &cx);
-  double num = sx * (s2 - s1) - sin(c * x) / ((1.0 + c) * x) + cx * (c2 - c1);
-  return num / (log(1.0 + c) - c / (1.0 + c));
+// Normalised Fourier transform u(k | m, c) of the truncated NFW profile
+// (200 x mean-density mass) with K = k r_vir, the concentration c and
+// l1 = ln(1 + c), inorm = 1 / (l1 - c / (1 + c)).  For c >= 1, with x = K / c:
+//   u inorm^-1 = sin x (Si(x + K) - Si(x)) + cos x (Ci(x + K) - Ci(x)) - sin K / (x + K).
+// The angle of the second argument minus that of the first is K, so where
+// x + K >= 4 the auxiliary functions leave
+//   g(x) + (f(x + K) - 1 / (x + K)) sin K - g(x + K) cos K,
+// with g(x) from its definition for x < 4; below, Ci(x + K) - Ci(x) is
+// ln(1 + c) plus two entire functions.  c < 1: the defining integral.
+__device__ __forceinline__ double dev_nfw_u(double K, double c, double l1, double inorm, const double* x16,
+                                            const double* w16) {
+  if (c < WL_NFW_C_INTEGRAL) return dev_nfw_u_integral(K, c, x16, w16);
+  const double x = K / c, x2 = x + K;
+  double sK, cK, num;
+  sincos(K, &sK, &cK);
+  const double i2 = 1.0 / x2;
+  if (x2 >= 4.0) {
+    double f2, g2, g1;
+    dev_sici_fg(x2, i2, &f2, &g2);
+    if (x >= 4.0) {
+      double f1;
+      dev_sici_fg(x, c / K, &f1, &g1);
+    } else {
+      double p, q, sx, cx;
+      dev_sici_small(x * x, &p, &q);
+      sincos(x, &sx, &cx);
+      g1 = (0.5 * WL_PI - x * p) * sx - (WL_EULER_GAMMA + log(x) + x * x * q) * cx;
+    }
+    num = g1 + (f2 - i2) * sK - g2 * cK;
+  } else {
+    double p1, q1, p2, q2, sx, cx;
+    dev_sici_small(x * x, &p1, &q1);
+    dev_sici_small(x2 * x2, &p2, &q2);
+    sincos(x, &sx, &cx);
+    num = sx * (x2 * p2 - x * p1) + cx * (l1 + (x2 * x2 * q2 - x * x * q1)) - sK * i2;
+  }
+  return num * inorm;
 }
 
 template <typename T>
