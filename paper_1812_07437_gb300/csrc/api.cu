@@ -245,7 +245,9 @@ static void free_all(cov_handle* h) {
                   h->kap,   h->kgram, h->kcol,    h->kn,      h->koff,      h->plist,
                   h->knode, h->kwt,   h->kw8,     h->kws,     h->zsrc,      h->gsel,    h->cmass,   h->chebm,
                   h->trigeo, h->zint, h->pk,      h->amp_part, h->Draw,     h->chis,    h->cz,      h->rvir,
-                  h->hint,  h->qw,    h->proj,    h->ksum,    h->kticket};
+                  h->hint,  h->qw,    h->proj,    h->ksum,    h->kticket,
+                  h->Asl,   h->Tsl,   h->Aexp,    h->Texp,    h->trd,       h->sl_s2,   h->sl_w,    h->sl_sr,
+                  h->sl_part};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (h->tile_ring) cudaFree(h->tile_ring);
@@ -259,8 +261,9 @@ static void free_all(cov_handle* h) {
   if (h->batch_D) cudaFree(h->batch_D);
 }
 
-// Device tables that cov_init allocates for a planned handle (pointer, bytes).
-static void init_allocs(cov_handle* h, std::vector<std::pair<void**, size_t>>& al) {
+// Device tables that cov_init allocates for a planned handle (pointer, bytes);
+// returns the bytes of the builders' own tables among them.
+static size_t init_allocs(cov_handle* h, std::vector<std::pair<void**, size_t>>& al) {
   const size_t d = sizeof(double);
   size_t nl = h->nl, nt = h->nt, nchi = h->nchi, nm = h->nm, nmb = h->nmb, nc = h->nc;
   size_t ntri = std::max(h->ntri, 1);
@@ -293,6 +296,8 @@ static void init_allocs(cov_handle* h, std::vector<std::pair<void**, size_t>>& a
       {(void**)&h->B1h3, d * ntri * nchi},  {(void**)&h->Ps, d * nl * nt * nt},
       {(void**)&h->B1hp, d * ntri * nt * nt * nt},
       {(void**)&h->cosmo_d, sizeof(cov_cosmology)},
+  };
+  const std::vector<std::pair<void**, size_t>> builders = {
       {(void**)&h->knode, d * WL_N_K},      {(void**)&h->kwt, d * WL_N_K},
       {(void**)&h->kw8, d * WL_N_K},        {(void**)&h->kws, d * WL_N_K},
       {(void**)&h->pk, d * WL_N_K},         {(void**)&h->amp_part, d * (WL_N_K / WL_KT_THREADS)},
@@ -309,14 +314,22 @@ static void init_allocs(cov_handle* h, std::vector<std::pair<void**, size_t>>& a
       {(void**)&h->qw, d * (nt * (nt + 1) / 2 + nt * (nt + 1) * (nt + 2) / 6) * nchi},
       {(void**)&h->proj, d * (nl * (nt * (nt + 1) / 2) + ntri * (nt * (nt + 1) * (nt + 2) / 6))},
   };
+  size_t own = 0;
+  for (const auto& b : builders) {
+    al.push_back(b);
+    own += b.second;
+  }
+  return own;
 }
 
 // Host-only upper estimate of the device bytes one request holds at its peak:
 // the handle's tables, the dense covariance and data vector, the contraction
 // operands of the chosen precision, the trispectrum table, the Cholesky
-// workspace of the joint vector and the launch-order tables.  No CUDA call.
+// workspace of the joint vector and the launch-order tables.  digits: the FP64
+// form with its rows as digits (the tensor-core contraction) instead of FP64 rows.
+// No CUDA call.
 int wl_request_bytes(const cov_nz* nz, const cov_bins* bins, int precision, unsigned terms, int64_t* M_out,
-                     size_t* bytes) {
+                     size_t* bytes, bool digits) {
   cov_cosmology c0{0.31, 0.049, 0.68, 0.96, 0.83, -1.0, 2.7255};
   if (validate(&c0, nz, bins) != COV_OK) return COV_ERR_INVALID;
   cov_handle h;
@@ -324,15 +337,20 @@ int wl_request_bytes(const cov_nz* nz, const cov_bins* bins, int precision, unsi
   h.bins = *bins;
   plan(&h);
   std::vector<std::pair<void**, size_t>> al;
-  init_allocs(&h, al);
+  const size_t own = init_allocs(&h, al);
   size_t b = 0;
   for (auto& a : al) b += a.second;
   const size_t M = (size_t)h.M, K = (size_t)h.K, nchi = (size_t)h.nchi, nt = (size_t)h.ntrow;
   auto pad256 = [](size_t x) { return (x + 255) / 256 * 256; };
   auto kpad = [](size_t x) { return (x + 63) / 64 * 64; };
   b += M * M * 8 + M * 8;                                        // covariance, data vector
+  digits = digits && precision == COV_FP64;
+  if (digits && (terms & (COV_TERM_1H | COV_TERM_BBPT)))
+    b += wl_sl_fixed_bytes(&h);                                  // weights, exponents, shared partial sums
   if (terms & COV_TERM_1H) {
-    if (precision == COV_FP64)
+    if (digits)
+      b += wl_sl_bytes((int64_t)M, (int64_t)(K + nchi));         // digits of the factor and SSC rows
+    else if (precision == COV_FP64)
       b += M * K * 8 + M * nchi * 8;                             // FP64 factor and SSC rows
     else
       b += 2 * pad256(M) * kpad(K + nchi) * 2 + M * 8 + 16 * (K + nchi) +
@@ -340,7 +358,9 @@ int wl_request_bytes(const cov_nz* nz, const cov_bins* bins, int precision, unsi
   }
   if (terms & COV_TERM_BBPT) {
     b += nt * nt * 8;                                            // trispectrum table
-    if (precision == COV_FP64)
+    if (digits)
+      b += wl_sl_bytes((int64_t)nt, (int64_t)K);                 // digits of the trispectrum rows
+    else if (precision == COV_FP64)
       b += nt * K * 8;                                           // FP64 trispectrum rows
     else
       b += 2 * pad256(nt) * kpad(K) * 2 + nt * 8 +
@@ -351,7 +371,9 @@ int wl_request_bytes(const cov_nz* nz, const cov_bins* bins, int precision, unsi
   b += WL_TILE_CACHE * (t * (t + 1) / 2) * 8;                    // launch-order ring
   const size_t nb32 = (M + 31) / 32;
   if (terms & (COV_TERM_BBPT | COV_TERM_PB)) b += nb32 * (nb32 + 1) / 2 * 4;  // product-term block list (bound)
-  b += (size_t)64 << 20;                                         // small buffers, allocation granularity
+  // small buffers (the builders' tables among them), allocation granularity
+  const size_t small = (size_t)64 << 20;
+  b = b - own + std::max(small, own);
   *M_out = h.M;
   *bytes = b;
   return COV_OK;

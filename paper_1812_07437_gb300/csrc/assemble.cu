@@ -442,13 +442,26 @@ static int gauss(cov_handle* h, const GatherArgs& g, int64_t r0, int64_t r1, Out
   return COV_OK;
 }
 
-// The 1-halo trispectrum table T = R R^T of the PT term (Eq. CovBB): FP64
-// rows and an FP64 product, or BF16 hi/lo rows built straight from the bin
-// pair signatures and the tensor-core contraction.
+// The 1-halo trispectrum table T = R R^T of the PT term (Eq. CovBB): digit rows and
+// the exact-sum contraction (FP64 form; FP64 rows and an FP64 product where the
+// digits do not fit), or BF16 hi/lo rows built straight from the bin pair
+// signatures and the tensor-core contraction.  The FP64 form's caller resets and
+// checks the status word.
 static int build_ttable(cov_handle* h, int precision, cudaStream_t s) {
   int rc;
   const int64_t K = h->K;
   if ((rc = ensure(h, (void**)&h->Tmat, sizeof(double) * h->ntrow * h->ntrow, "trispectrum table"))) return rc;
+  bool digits = false;
+  if (precision == COV_FP64 && (rc = wl_sl_alloc(h, true, &digits, s))) return rc;
+  if (digits) {
+    int tk = wl_stage_begin(h, ST_ROWS_T, s);
+    if ((rc = wl_sl_rows(h, true, 0, s))) return rc;
+    wl_stage_end(h, tk, s);
+    tk = wl_stage_begin(h, ST_SYRK_T, s);
+    if ((rc = wl_sl_syrk(h, true, 0, out_rows(h->Tmat, h->ntrow), h->ntrow, s))) return rc;
+    wl_stage_end(h, tk, s);
+    return COV_OK;
+  }
   if (precision == COV_FP64) {
     if ((rc = ensure(h, (void**)&h->Trows, sizeof(double) * h->ntrow * K, "trispectrum rows"))) return rc;
     int tk = wl_stage_begin(h, ST_ROWS_T, s);
@@ -479,13 +492,26 @@ static int build_ttable(cov_handle* h, int precision, cudaStream_t s) {
 int wl_assemble(cov_handle* h, double* C, int64_t ldc, unsigned terms, int precision, cudaStream_t s) {
   int rc;
   const int64_t M = h->M, K = h->K;
-  bool ssc_merged = false;
+  bool ssc_merged = false, digits = false;
+  const bool fp64 = precision == COV_FP64;
+  if (fp64 && (terms & (COV_TERM_1H | COV_TERM_BBPT)) && (rc = wl_tc_status_reset(h, s))) return rc;
   // 1. the 1-halo trispectrum table of the PT term
   if (terms & COV_TERM_BBPT)
     if ((rc = build_ttable(h, precision, s))) return rc;
   // 2. 1-halo (chi, M) contraction: the first writer of the lower triangle
   if (terms & COV_TERM_1H) {
-    if (precision == COV_FP64) {
+    if (fp64 && (rc = wl_sl_alloc(h, false, &digits, s))) return rc;
+    if (digits) {
+      // the super-sample rows ride along as N_chi extra columns
+      ssc_merged = (terms & COV_TERM_SSC) != 0;
+      const int nssc = ssc_merged ? h->nchi : 0;
+      int tk = wl_stage_begin(h, ST_ROWS_A, s);
+      if ((rc = wl_sl_rows(h, false, nssc, s))) return rc;
+      wl_stage_end(h, tk, s);
+      tk = wl_stage_begin(h, ST_SYRK_1H, s);
+      if ((rc = wl_sl_syrk(h, false, nssc, out_rows(C, ldc), M, s))) return rc;
+      wl_stage_end(h, tk, s);
+    } else if (fp64) {
       if ((rc = ensure(h, (void**)&h->A, sizeof(double) * M * K, "FP64 factor rows"))) return rc;
       int tk = wl_stage_begin(h, ST_ROWS_A, s);
       if ((rc = wl_rows_a(h, s))) return rc;
@@ -537,6 +563,8 @@ int wl_assemble(cov_handle* h, double* C, int64_t ldc, unsigned terms, int preci
       return rc;
     wl_stage_end(h, tk, s);
   }
+  if (fp64 && (h->sl_rows > 0 || h->sl_tri > 0) && (terms & (COV_TERM_1H | COV_TERM_BBPT)))
+    return wl_tc_status_check(h, s);
   return COV_OK;
 }
 
@@ -549,7 +577,13 @@ static int prepare_operands(cov_handle* h, unsigned terms, int precision, cudaSt
   const int64_t M = h->M, K = h->K;
   if (terms & COV_TERM_BBPT)
     if ((rc = build_ttable(h, precision, s))) return rc;
-  if (precision == COV_FP64) {
+  bool digits = false;
+  if (precision == COV_FP64 && (terms & COV_TERM_1H) && (rc = wl_sl_alloc(h, false, &digits, s))) return rc;
+  if (digits) {
+    int tk = wl_stage_begin(h, ST_ROWS_A, s);
+    if ((rc = wl_sl_rows(h, false, (terms & COV_TERM_SSC) ? h->nchi : 0, s))) return rc;
+    wl_stage_end(h, tk, s);
+  } else if (precision == COV_FP64) {
     if (terms & COV_TERM_1H) {
       if ((rc = ensure(h, (void**)&h->A, sizeof(double) * M * K, "FP64 factor rows"))) return rc;
       int tk = wl_stage_begin(h, ST_ROWS_A, s);
@@ -589,6 +623,7 @@ static int prepare_operands(cov_handle* h, unsigned terms, int precision, cudaSt
 int wl_assemble_band(cov_handle* h, int64_t row0, int64_t nrows, OutMap out, unsigned terms, int precision,
                      cudaStream_t s) {
   int rc;
+  if (precision == COV_FP64 && (terms & (COV_TERM_1H | COV_TERM_BBPT)) && (rc = wl_tc_status_reset(h, s))) return rc;
   if (h->ops_terms != (int)terms || h->ops_precision != precision) {
     if ((rc = prepare_operands(h, terms, precision, s))) return rc;
     h->ops_terms = (int)terms;
@@ -645,9 +680,15 @@ int wl_assemble_band(cov_handle* h, int64_t row0, int64_t nrows, OutMap out, uns
     return wl_tc_status_check(h, s);
   }
   // FP64 form, or no 1-halo term: contraction, products, super-sample term in turn
+  // (the digit form's contraction holds the super-sample columns)
+  const bool digits = precision == COV_FP64 && h->sl_rows > 0;
   if (terms & COV_TERM_1H) {
     int tk = wl_stage_begin(h, ST_SYRK_1H, s);
-    if ((rc = gemm_lower_band(h, h->A, h->K, row1, h->K, 0.0, out, s))) return rc;
+    if (digits) {
+      if ((rc = wl_sl_syrk(h, false, (terms & COV_TERM_SSC) ? h->nchi : 0, out, row1, s))) return rc;
+    } else if ((rc = gemm_lower_band(h, h->A, h->K, row1, h->K, 0.0, out, s))) {
+      return rc;
+    }
     wl_stage_end(h, tk, s);
   }
   int tg = wl_stage_begin(h, ST_GATHER, s);
@@ -655,10 +696,12 @@ int wl_assemble_band(cov_handle* h, int64_t row0, int64_t nrows, OutMap out, uns
   WL_LAUNCH(h, "k_gather");
   if ((rc = gauss(h, g, row0, row1, out, s))) return rc;
   wl_stage_end(h, tg, s);
-  if ((terms & COV_TERM_SSC) && (terms & COV_TERM_1H)) {
+  if ((terms & COV_TERM_SSC) && (terms & COV_TERM_1H) && !digits) {
     int tk = wl_stage_begin(h, ST_SYRK_SSC, s);
     if ((rc = gemm_lower_band(h, h->Srows, h->nchi, row1, h->nchi, 1.0, out, s))) return rc;
     wl_stage_end(h, tk, s);
   }
+  if (precision == COV_FP64 && (digits || h->sl_tri > 0) && (terms & (COV_TERM_1H | COV_TERM_BBPT)))
+    return wl_tc_status_check(h, s);
   return COV_OK;
 }

@@ -193,27 +193,6 @@ __device__ __forceinline__ double scaled_to_double(long long a, int ex) {
   return __longlong_as_double((long long)(sign | ((unsigned long long)e << 52) | (m & ((1ull << 52) - 1))));
 }
 
-// RN(a) 2^ex as an FP64 value for 0 < |a| < 2^63, without branches on the
-// value: normalise |a| so that its leading bit is bit 63, keep the 53 leading
-// bits rounded to nearest (ties to even), and add the rounded significand
-// (2^52 <= r <= 2^53) to the biased exponent field, which carries a rounding
-// overflow into the exponent by itself.  Results outside the normal range take
-// the FP64 path.
-__device__ __forceinline__ double scaled_to_double_rn(long long a, int ex) {
-  if (a == 0) return 0.0;
-  const unsigned long long sign = (unsigned long long)a & (1ull << 63);
-  const unsigned long long u = a < 0 ? 0ull - (unsigned long long)a : (unsigned long long)a;
-  const int lz = __clzll((long long)u);
-  const unsigned long long mn = u << lz;
-  const unsigned long long r0 = mn >> 11;
-  const unsigned long long rb = (mn >> 10) & 1ull;
-  const unsigned long long sticky = ((mn & 0x3FFull) != 0ull) | (r0 & 1ull);
-  const unsigned long long r = r0 + (rb & sticky);
-  const int e = (63 - lz) + ex + 1023;
-  if (e <= 0 || e >= 2046) return ldexp((double)a, ex);
-  return __longlong_as_double((long long)(sign | (((unsigned long long)(e - 1) << 52) + r)));
-}
-
 // Lower tiles of one update launch, row by row: tile row ti (128 rows, from
 // ti0 = tj0 * 64 / 128) holds the column tiles tj0 .. min(tj0 + ntj - 1,
 // 2 ti + 1) (64 columns each).  cum(ti) counts the tiles of rows ti0 .. ti-1.
@@ -751,6 +730,20 @@ __global__ void __launch_bounds__(PU_THREADS, 1)
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
 }
 
+int wl_num_sms() {
+  static std::once_flag once[WL_MAX_DEVICES];
+  static int n[WL_MAX_DEVICES];
+  int d = 0;
+  cudaGetDevice(&d);
+  if (d < 0 || d >= WL_MAX_DEVICES) return 1;
+  std::call_once(once[d], [&] {
+    n[d] = 1;
+    cudaDeviceGetAttribute(&n[d], cudaDevAttrMultiProcessorCount, d);
+    if (n[d] < 1) n[d] = 1;
+  });
+  return n[d];
+}
+
 static PFN_cuTensorMapEncodeTiled_v12000 cs_encode() { return wl_encode_tiled(); }
 
 static int cs_map(cov_handle* h, CUtensorMap* map, void* base, int64_t total_rows, int box_rows) {
@@ -853,20 +846,6 @@ static bool pu_usable(const cov_handle* h, const OutMap& W) {
   return W.tiled || (W.ldc % 2 == 0);
 }
 
-static int pu_num_sms() {
-  static std::once_flag once[WL_MAX_DEVICES];
-  static int n[WL_MAX_DEVICES];
-  int d = 0;
-  cudaGetDevice(&d);
-  if (d < 0 || d >= WL_MAX_DEVICES) return 1;
-  std::call_once(once[d], [&] {
-    n[d] = 1;
-    cudaDeviceGetAttribute(&n[d], cudaDevAttrMultiProcessorCount, d);
-    if (n[d] < 1) n[d] = 1;
-  });
-  return n[d];
-}
-
 // slices of the panel rows r0..r1-1, columns k0..k0+kb-1 of the workspace
 int wl_chol_slice(cov_handle* h, OutMap W, int64_t k0, int kb, int64_t r0, int64_t r1, void* buf, cudaStream_t s) {
   int64_t n = r1 - r0;
@@ -954,7 +933,7 @@ static int pu_update(cov_handle* h, OutMap W, int64_t r0, int64_t r1, const void
         return (int)cudaFuncSetAttribute(k_chol_upd, cudaFuncAttributeMaxDynamicSharedMemorySize, PU_SMEM);
       }) != 0)
     return wl_fail(h, COV_ERR_CUDA, "cudaFuncSetAttribute(k_chol_upd) failed");
-  const int64_t grid = std::min<int64_t>(pu_num_sms(), nt);
+  const int64_t grid = std::min<int64_t>(wl_num_sms(), nt);
   k_chol_upd<<<(unsigned)grid, PU_THREADS, PU_SMEM, s>>>(mi, mj, mc, rexp, u, status);
   WL_LAUNCH(h, "k_chol_upd");
   return COV_OK;

@@ -211,6 +211,14 @@ struct cov_handle {
   uint16_t *Thi = nullptr, *Tlo = nullptr;  // split trispectrum rows (tensor-core form)
   double* Tscale = nullptr;
   double* Srows = nullptr;  // [M][nchi]
+  // FP64 form on the tensor cores: digit blocks and row exponents of the factor rows
+  // and the trispectrum rows, the latter's descriptors, and their builders' tables
+  uint8_t *Asl = nullptr, *Tsl = nullptr;
+  int *Aexp = nullptr, *Texp = nullptr;
+  int32_t* trd = nullptr;
+  double *sl_s2 = nullptr, *sl_w = nullptr, *sl_sr = nullptr;
+  unsigned long long* sl_part = nullptr;  // exact partial sums of tiles shared by several CTAs, then their tickets
+  int sl_rows = 0, sl_tri = 0;            // 0 undecided, 1 digits, -1 FP64 rows (k_gemm_lower)
   double* work = nullptr;   // Cholesky workspace (M+1) rows
   int64_t work_n = 0;
   int64_t work_ld = 0;      // its row length (the last dense cov_snr)
@@ -287,12 +295,18 @@ int wl_gemm_lower_fp64(cov_handle* h, const double* A, int64_t lda, const double
                        cudaStream_t s);  // assemble.cu
 int wl_syrk_tc(cov_handle* h, int nssc, OutMap out, cudaStream_t s, int64_t row1 = -1);  // syrk_tc.cu
 int wl_syrk_tc_part(cov_handle* h, int nssc, OutMap out, int64_t r0, int64_t r1, cudaStream_t s);
+int wl_num_sms();  // chol_tc.cu: SMs of the current device
+size_t wl_sl_bytes(int64_t rows, int64_t k);                                             // syrk_sl.cu
+size_t wl_sl_fixed_bytes(const cov_handle* h);                                           // syrk_sl.cu
+int wl_sl_alloc(cov_handle* h, bool tri, bool* use, cudaStream_t s);                     // syrk_sl.cu
+int wl_sl_rows(cov_handle* h, bool tri, int nssc, cudaStream_t s);                       // syrk_sl.cu
+int wl_sl_syrk(cov_handle* h, bool tri, int nssc, OutMap out, int64_t row1, cudaStream_t s);  // syrk_sl.cu
 int wl_tc_status_reset(cov_handle* h, cudaStream_t s);
 int wl_tc_status_check(cov_handle* h, cudaStream_t s);
 int wl_split_bytes(int64_t M, int K, size_t* bytes);                      // syrk_tc.cu
 int wl_kpad(int K);  // K padded to the contraction's K granularity
 int wl_request_bytes(const cov_nz* nz, const cov_bins* bins, int precision, unsigned terms, int64_t* M,
-                     size_t* bytes);  // api.cu: host-only footprint estimate of one request
+                     size_t* bytes, bool digits = false);  // api.cu: host-only footprint estimate of one request
 size_t wl_handle_bytes(const cov_handle* h);
 void wl_set_global_error(const std::string& msg);  // api.cu: read by cov_last_error(NULL)
 size_t wl_chol_tc_bytes(int64_t n);  // chol_tc.cu
@@ -542,6 +556,27 @@ __device__ __forceinline__ double dev_nfw_u(double K, double c, double l1, doubl
     num = sx * (x2 * p2 - x * p1) + cx * (l1 + (x2 * x2 * q2 - x * x * q1)) - sK * i2;
   }
   return num * inorm;
+}
+
+// RN(a) 2^ex as an FP64 value for 0 < |a| < 2^63, without branches on the
+// value: normalise |a| so that its leading bit is bit 63, keep the 53 leading
+// bits rounded to nearest (ties to even), and add the rounded significand
+// (2^52 <= r <= 2^53) to the biased exponent field, which carries a rounding
+// overflow into the exponent by itself.  Results outside the normal range take
+// the FP64 path.
+__device__ __forceinline__ double scaled_to_double_rn(long long a, int ex) {
+  if (a == 0) return 0.0;
+  const unsigned long long sign = (unsigned long long)a & (1ull << 63);
+  const unsigned long long u = a < 0 ? 0ull - (unsigned long long)a : (unsigned long long)a;
+  const int lz = __clzll((long long)u);
+  const unsigned long long mn = u << lz;
+  const unsigned long long r0 = mn >> 11;
+  const unsigned long long rb = (mn >> 10) & 1ull;
+  const unsigned long long sticky = ((mn & 0x3FFull) != 0ull) | (r0 & 1ull);
+  const unsigned long long r = r0 + (rb & sticky);
+  const int e = (63 - lz) + ex + 1023;
+  if (e <= 0 || e >= 2046) return ldexp((double)a, ex);
+  return __longlong_as_double((long long)(sign | (((unsigned long long)(e - 1) << 52) + r)));
 }
 
 template <typename T>

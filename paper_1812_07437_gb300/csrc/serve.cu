@@ -41,6 +41,7 @@ struct Rec {
   std::vector<double> snr;
   std::string key, err;
   int bypassed = 0;
+  bool digits = false;  // the reservation holds the FP64 form's digit rows
 };
 
 std::string key_of(const cov_request& r) {
@@ -165,6 +166,8 @@ static int run_request(cov_server* s, Rec& q, Resident* res, cudaStream_t stream
       q.err = cov_last_error(nullptr);
       return rc;
     }
+    // the FP64 form's digits only where the reservation holds them
+    if (!q.digits) res->h->sl_rows = res->h->sl_tri = -1;
     const size_t M = (size_t)res->h->M;
     if (cudaMalloc(&res->C, sizeof(double) * M * M) != cudaSuccess ||
         cudaMalloc(&res->D, sizeof(double) * M) != cudaSuccess) {
@@ -336,6 +339,14 @@ extern "C" int cov_server_submit(cov_server* s, const cov_request* r, int64_t* i
     s->recs.emplace(*id, std::move(q));
     s->cv_done.notify_all();
     return COV_OK;
+  }
+  if (s->o.precision == COV_FP64 && s->o.dry_run_us <= 0) {
+    // the tensor-core FP64 form where its larger rows fit the budget, else the FP64 rows
+    int64_t M = 0;
+    size_t with = 0;
+    q.digits = wl_request_bytes(&r->nz, &r->bins, COV_FP64, s->o.terms, &M, &with, true) == COV_OK &&
+               with <= s->o.hbm_budget;
+    if (q.digits) q.info.footprint = std::max(q.info.footprint, with);
   }
   if (q.info.footprint > s->o.hbm_budget) {
     q.info.state = COV_REQ_REJECTED;
