@@ -51,7 +51,7 @@ extern "C" {
  * has eigenvalues near that (strongly overlapping tomographic kernels, e.g. no
  * photo-z scatter and several bins) can then lose positive definiteness and
  * the S/N returns COV_ERR_NOT_PD: assemble such covariances in COV_FP64. */
-#define COV_FP64 0       /* plain FP64 on CUDA cores                          */
+#define COV_FP64 0       /* FP64 accuracy: exact digit sums (tensor cores)    */
 #define COV_SPLIT_BF16 1 /* tcgen05 tensor cores, A = hi + lo in BF16, FP32 acc */
 
 /* selection for the signal-to-noise (Sec. 5, Eq. eq:SN2) */
@@ -122,9 +122,9 @@ typedef struct {
                      /* where 2-CTA clusters fit) or COV_TC_SINGLE (one CTA   */
                      /* per 256 x 256 tile); both give the same sums          */
   int chol_kernel;   /* Cholesky trailing update (cov_snr, cov_snr_tiles):    */
-                     /* COV_CHOL_AUTO (persistent, 128 x 32 tiles, epilogue   */
-                     /* overlapping the next tile's MMAs) or COV_CHOL_TILE    */
-                     /* (one CTA per 128 x 64 tile); bit-identical results    */
+                     /* COV_CHOL_AUTO (persistent, 128 x 64 tiles, the next   */
+                     /* tile's loads under the epilogue) or COV_CHOL_TILE     */
+                     /* (one CTA per tile); bit-identical results             */
   int coupling;      /* coupling of the BB+PT terms (Eq. CovBB):             */
                      /* COV_COUPLING_MODES: 1/N(l^b) with the exact mode     */
                      /* count, the paper's prefactor 2 pi/(Omega l Delta l)  */

@@ -322,6 +322,13 @@ static size_t init_allocs(cov_handle* h, std::vector<std::pair<void**, size_t>>&
   return own;
 }
 
+// Half of the Cholesky scratch that the estimate below reserves for n rows (the scratch
+// itself adapts to twice this and some slack, see cov_handle::chol_scratch_cap)
+size_t wl_chol_scratch_est(int64_t n) {
+  const size_t pad = (size_t)(n + 64 + 127) / 128 * 128;
+  return (pad * 772 + 255) / 256 * 256;
+}
+
 // Host-only upper estimate of the device bytes one request holds at its peak:
 // the handle's tables, the dense covariance and data vector, the contraction
 // operands of the chosen precision, the trispectrum table, the Cholesky
@@ -366,7 +373,7 @@ int wl_request_bytes(const cov_nz* nz, const cov_bins* bins, int precision, unsi
       b += 2 * pad256(nt) * kpad(K) * 2 + nt * 8 +
            (size_t)h.nl * (h.nl + 1) / 2 * (K * 4 + nchi * 12);   // BF16 rows, pair signatures
   }
-  b += (M + 8) * (M + 1) * 8 + 2 * ((wl_chol_tc_bytes((int64_t)M + 1) + 255) / 256 * 256) + M * 4;
+  b += (M + 8) * (M + 1) * 8 + 2 * wl_chol_scratch_est((int64_t)M + 1) + M * 4;
   size_t t = (std::max(M, nt) + 255) / 256 + 1;
   b += WL_TILE_CACHE * (t * (t + 1) / 2) * 8;                    // launch-order ring
   const size_t nb32 = (M + 31) / 32;

@@ -224,8 +224,9 @@ struct cov_handle {
   int64_t work_ld = 0;      // its row length (the last dense cov_snr)
   void* pca_buf = nullptr;  // PCA: G, y and the per-mode arrays
   size_t pca_bytes = 0;
-  void* chol_scratch = nullptr;  // two slice buffers of the tensor-core trailing update
+  void* chol_scratch = nullptr;  // Cholesky: digit buffers, diagonal factors, data vector, scaling
   size_t chol_scratch_n = 0;
+  size_t chol_scratch_cap = 0;   // bytes it should stay within (the server's reservation; 0: no limit)
   cudaStream_t side = nullptr;   // look-ahead stream of the Cholesky panel kernels
   cudaEvent_t ev_cols = nullptr, ev_panel = nullptr;
   int* chol_status = nullptr;
@@ -234,7 +235,7 @@ struct cov_handle {
   cov_cosmology* cosmo_d = nullptr;  // the cosmology the kernels read (device copy of cosmo)
   bool deferred = false;  // inside a captured batch step: no host synchronisation, no host-side copies
   bool chol_lookahead = true;  // Cholesky panel look-ahead on the side stream
-  int chol_kernel = 0;         // Cholesky trailing update: 0 persistent (k_chol_upd), 1 one CTA per tile
+  int chol_kernel = 0;         // Cholesky trailing update: 0 persistent CTAs, 1 one CTA per tile
   int tc_kernel = -1;          // contraction kernel: -1 automatic, 0 one CTA per tile, 1 CTA pairs
   int pr_group = 8;            // tile rows per group of the pair-tile launch order
   struct Selection {           // cumulative S/N selections (P, B, joint; all rows in place)
@@ -295,7 +296,7 @@ int wl_gemm_lower_fp64(cov_handle* h, const double* A, int64_t lda, const double
                        cudaStream_t s);  // assemble.cu
 int wl_syrk_tc(cov_handle* h, int nssc, OutMap out, cudaStream_t s, int64_t row1 = -1);  // syrk_tc.cu
 int wl_syrk_tc_part(cov_handle* h, int nssc, OutMap out, int64_t r0, int64_t r1, cudaStream_t s);
-int wl_num_sms();  // chol_tc.cu: SMs of the current device
+int wl_num_sms();  // chol_fx.cu: SMs of the current device
 size_t wl_sl_bytes(int64_t rows, int64_t k);                                             // syrk_sl.cu
 size_t wl_sl_fixed_bytes(const cov_handle* h);                                           // syrk_sl.cu
 int wl_sl_alloc(cov_handle* h, bool tri, bool* use, cudaStream_t s);                     // syrk_sl.cu
@@ -309,14 +310,11 @@ int wl_request_bytes(const cov_nz* nz, const cov_bins* bins, int precision, unsi
                      size_t* bytes, bool digits = false);  // api.cu: host-only footprint estimate of one request
 size_t wl_handle_bytes(const cov_handle* h);
 void wl_set_global_error(const std::string& msg);  // api.cu: read by cov_last_error(NULL)
-size_t wl_chol_tc_bytes(int64_t n);  // chol_tc.cu
-int wl_chol_slice(cov_handle* h, OutMap W, int64_t k0, int kb, int64_t r0, int64_t r1, void* buf, cudaStream_t s);
-bool wl_chol_fused_panel(const cov_handle* h, const OutMap& W);  // chol_tc.cu
+size_t wl_chol_scratch_est(int64_t n);  // api.cu
+size_t wl_fx_bytes(int64_t n, int w);  // chol_fx.cu: scratch with super-panels of w panels
+int wl_fx_factor(cov_handle* h, OutMap W, int64_t Ms, const int* perm, const double* C, int64_t ldc, const double* D,
+                 cudaStream_t s);  // chol_fx.cu
 int wl_side_stream(cov_handle* h);  // api.cu: the handle's high-priority side stream
-int wl_chol_trsm_slice(cov_handle* h, OutMap W, int64_t k0, int kb, int64_t r0, int64_t r1, void* buf,
-                       cudaStream_t s);
-int wl_chol_update(cov_handle* h, OutMap W, int64_t r0, int64_t r1, const void* buf, int tj0, int ntj, int* status,
-                   cudaStream_t s);
 int wl_syrk_tc_rows(cov_handle* h, const void* hi, const void* lo, const double* rscale, int64_t rows, int Kp,
                     OutMap out, cudaStream_t s, int64_t row1 = -1);
 // ---- device helpers ------------------------------------------------------------

@@ -169,6 +169,7 @@ static int run_request(cov_server* s, Rec& q, Resident* res, cudaStream_t stream
     // the FP64 form's digits only where the reservation holds them
     if (!q.digits) res->h->sl_rows = res->h->sl_tri = -1;
     const size_t M = (size_t)res->h->M;
+    res->h->chol_scratch_cap = 2 * wl_chol_scratch_est((int64_t)M + 1) + ((size_t)48 << 20);
     if (cudaMalloc(&res->C, sizeof(double) * M * M) != cudaSuccess ||
         cudaMalloc(&res->D, sizeof(double) * M) != cudaSuccess) {
       cudaGetLastError();

@@ -8,18 +8,10 @@
 //     2-norm below sqrt(2) (k_sl_norm), rounded to x = X 2^-55 with an integer X,
 //     and cut into the seven balanced base-256 digits of X: x = sum_t d_t 2^(-7-8t),
 //     |d_0| <= 182, |d_t| <= 128, each exact in BF16 (k_sl_rows).
-//   * Products.  d_t(i) d_u(j) and their sums over a K block of 32 at equal
-//     t + u = g, g = 0..6, stay below 2^22: exact in the FP32 accumulators.  The 28
-//     pairs t + u <= 6 are formed by 7 MMAs per K step instead of 28: the J digits
-//     u = 0..6 of a group of 32 columns are stacked in shared memory, the accumulators
-//     of the seven levels lie side by side in TMEM, and one MMA of digit t against the
-//     first 32 (7 - t) stacked rows lands on the levels t..6 (N = 224, 192, ..., 32).
-//     Small-N MMAs would read the 4 KB of the I digit from shared memory for 8 cycles
-//     of work each.
-//   * Recombination.  The level sums of a K block are added exactly to one 64-bit
-//     integer per element, sum_g a_g 2^(8 (6 - g)), modulo 2^64.  By Cauchy-Schwarz the
-//     complete sum is below 2^63 (that is what the norm scaling is for), so partial
-//     sums may wrap and need no second word.  One rounding to FP64 at the end.
+//   * Products and recombination as described in digits.cuh, modulo 2^64.  By
+//     Cauchy-Schwarz the complete sum is below 2^63 (that is what the norm scaling is
+//     for), so partial sums may wrap and need no second word.  One rounding to FP64 at
+//     the end.
 // What is dropped (levels above 6, digits beyond 2^-55 of the norm) is ~1e-15 of
 // sqrt(C_aa C_bb); against extended precision on the paper's and the 5-bin rows the
 // error is 0.8-1.4e-15 in the 2-norm where the FP64 FMA chain of k_gemm_lower, one
@@ -28,28 +20,12 @@
 //
 // Bound: the tensor pipe and, close behind, L2 (a 128 x 128 tile reads 112 KB per K
 // block of 32, 32 bytes per clock and SM at the full MMA rate).  M = 6375, K = 12288 +
-// 128: contraction 10.7 ms = 1.36 PFLOP/s issued (48 TFLOP/s FP64) where k_gemm_lower
+// 128: contraction 10.0 ms = 1.45 PFLOP/s issued (51 TFLOP/s FP64) where k_gemm_lower
 // took 415 + 4.4 ms (1.2 TFLOP/s); trispectrum table 37 -> 1.0 ms, rows 0.55 ms; whole
-// FP64 assembly 464 -> 12.6 ms.  M = 818 (28 tiles, 11 K parts each): 27.2 -> 0.65 ms.
-#include <cuda_bf16.h>
+// FP64 assembly 464 -> 11.8 ms.  M = 818 (28 tiles, 11 K parts each): 27.1 -> 0.63 ms.
+#include "digits.cuh"
 
-#include "common.cuh"
-
-#define SL_S 7
-#define SL_BM 128                                   // tile rows, and tile columns
-#define SL_BK 32                                    // K block
-#define SL_BN 32                                    // columns per accumulator group
-#define SL_NG (SL_BM / SL_BN)
-#define SL_DIGIT (SL_BM * SL_BK * 2)                // 8 KB: one digit of 128 rows x 32 K
-#define SL_BLOCK (SL_S * SL_DIGIT)                  // 56 KB: one (row block, K block)
-#define SL_GROUP (SL_S * SL_BN * SL_BK * 2)         // 14 KB: the digits of 32 rows
-#define SL_STAGE (SL_BLOCK + SL_NG * SL_GROUP)      // 112 KB
-#define SL_STAGES 2
-#define SL_SMEM (SL_STAGES * SL_STAGE + 1024)
-#define SL_EPI 8                                    // epilogue warps: two per TMEM lane quarter, 16 columns each
-#define SL_THREADS (64 + 32 * SL_EPI)
-#define SL_SPIN (1u << 22)
-#define SL_MAGIC 0x4B400000u                        // bits of 1.5 2^23: f + 1.5 2^23 holds the integer f in its low bits
+#define SL_NG 4               // a tile is 128 x 128
 #define SL_SPLIT_TILES 304                          // largest tile count whose K range is cut over several CTAs
 
 __global__ void k_rows_prep(int nchi, int nm, double inv_omega, const cov_cosmology* __restrict__ cosmo_p,
@@ -172,25 +148,6 @@ __global__ void __launch_bounds__(256) k_sl_norm(SlSig g, int64_t rows, const in
   if (lane == 0) rexp[a] = e;
 }
 
-// X = RN(x 2^55) (ties to even) for |x| < 2, by integer operations on the bits of x
-__device__ __forceinline__ long long sl_int(double x) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const int E = (int)((b >> 52) & 0x7FFu);
-  const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);  // (subnormals round to 0 either way)
-  const int sh = 1020 - E;  // X = RN(m / 2^sh); sh >= -3
-  unsigned long long q;
-  if (sh <= 0) {
-    q = m << -sh;
-  } else if (sh >= 64) {
-    q = 0;
-  } else {
-    q = m >> sh;
-    const unsigned long long rem = m & ((1ull << sh) - 1), half = 1ull << (sh - 1);
-    q += (rem > half || (rem == half && (q & 1ull))) ? 1ull : 0ull;
-  }
-  return (b >> 63) ? -(long long)q : (long long)q;
-}
-
 // Digits of 128 rows x 32 K, one contiguous 56 KB block per (row block, K block):
 // [digit][row][k].  The factor of each signature present among the rows is formed
 // once in shared memory; an entry is then one FP64 product (the bound here beside the
@@ -246,107 +203,33 @@ __global__ void __launch_bounds__(SR_THREADS)
     const int64_t r = r0 + row;
     const double* wr = wrow + r * g.nchi;
     const double* sr = srow + r * g.nchi;
-    uint32_t d[SL_S][4];
+    long long X[8];
+    uint4 d[SL_S];
     int n = (int)((k0 + k8) / g.nm), q = (int)((k0 + k8) % g.nm);
 #pragma unroll
-    for (int p = 0; p < 4; ++p) {
-      unsigned long long y[2];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int64_t kk = k0 + k8 + 2 * p + h;
-        double v = 0.0;
-        if (r < rows) {
-          if (kk < K)
-            v = F[slot[row]][k8 + 2 * p + h] * wr[n];
-          else if (kk < K + nssc)
-            v = sr[kk - K];
-        }
-        if (++q == g.nm) {
-          q = 0;
-          ++n;
-        }
-        // balanced digits d_t = byte_t(X + 128 sum_t 256^t) - 128
-        y[h] = (unsigned long long)sl_int(v) + 0x0080808080808080ull;
+    for (int p = 0; p < 8; ++p) {
+      const int64_t kk = k0 + k8 + p;
+      double v = 0.0;
+      if (r < rows) {
+        if (kk < K)
+          v = F[slot[row]][k8 + p] * wr[n];
+        else if (kk < K + nssc)
+          v = sr[kk - K];
       }
-#pragma unroll
-      for (int t = 0; t < SL_S; ++t) {
-        float f[2];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          // the top digit keeps its sign and ninth bit
-          const int by = t == 0 ? (int)((long long)y[h] >> 48) : (int)((y[h] >> (8 * (SL_S - 1 - t))) & 255u);
-          f[h] = __int_as_float(SL_MAGIC + by) - (12582912.0f + 128.0f);
-        }
-        // |d| <= 256 has at most 8 significant bits: the upper half of the FP32 value is its BF16 form
-        d[t][p] = __byte_perm(__float_as_uint(f[0]), __float_as_uint(f[1]), 0x7632);
+      if (++q == g.nm) {
+        q = 0;
+        ++n;
       }
+      X[p] = sl_int(v);
     }
+    sl_digits8(X, d);
 #pragma unroll
     for (int t = 0; t < SL_S; ++t)
-      *(uint4*)(o + (size_t)t * SL_DIGIT + row * (SL_BK * 2) + k8 * 2) = make_uint4(d[t][0], d[t][1], d[t][2], d[t][3]);
+      *(uint4*)(o + (size_t)t * SL_DIGIT + row * (SL_BK * 2) + k8 * 2) = d[t];
   }
 }
 
 // ---------------------------------------------------------------- contraction
-__device__ __forceinline__ uint32_t sl_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void sl_init(uint64_t* bar, uint32_t n) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(sl_u32(bar)), "r"(n) : "memory");
-}
-__device__ __forceinline__ void sl_expect(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(sl_u32(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void sl_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(sl_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void sl_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(sl_u32(bar))
-               : "memory");
-}
-__device__ __forceinline__ uint32_t sl_try(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(sl_u32(bar)), "r"(parity)
-      : "memory");
-  return ok;
-}
-// bounded wait that also gives up once any CTA has raised the status word
-__device__ __forceinline__ bool sl_wait(uint64_t* bar, uint32_t parity, int* status) {
-  for (uint32_t i = 0; i < SL_SPIN; ++i) {
-    if (sl_try(bar, parity)) return true;
-    if ((i & 1023u) == 1023u && *(volatile int*)status) return false;
-  }
-  atomicExch(status, 1);
-  return false;
-}
-__device__ __forceinline__ void sl_tma(const CUtensorMap* map, uint64_t* bar, void* dst, int row, int blk) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], "
-      "[%2];" ::"r"(sl_u32(dst)),
-      "l"((uint64_t)map), "r"(sl_u32(bar)), "r"(0), "r"(row), "r"(0), "r"(blk)
-      : "memory");
-}
-__device__ __forceinline__ void sl_prefetch(const CUtensorMap* map, int row, int blk) {
-  asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global.tile [%0, {%1, %2, %3, %4}];" ::"l"((uint64_t)map), "r"(0),
-               "r"(row), "r"(0), "r"(blk)
-               : "memory");
-}
-__device__ __forceinline__ uint64_t sl_desc(uint32_t saddr) {  // K-major, 64-byte rows, SWIZZLE_64B
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFF);
-  d |= (uint64_t)1 << 16;
-  d |= (uint64_t)(512 >> 4) << 32;  // 8 rows x 64 B
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)4 << 61;
-  return d;
-}
-__device__ __forceinline__ void sl_tmem_ld8(uint32_t taddr, uint32_t* r) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(taddr));
-}
-
 // Launch order of the lower 128 x 128 tiles of tile rows [t0, t1): groups of 8 tile
 // rows, column by column inside a group, so that the CTAs of a wave share few row
 // and column blocks in L2.
@@ -391,17 +274,14 @@ struct SlArgs {
 // One CTA per (128 x 128 lower tile, K range).  Warp 0 loads (TMA, two stages of a K
 // block: the I block in one box, the J block as four groups of 32 rows), warp 1 issues
 // the MMAs of the four column groups in turn into two accumulator sets (7 x 32
-// columns each), eight warps recombine the set of the group before: 14 integer and
-// FP32 operations per element and K block, in registers (64 64-bit sums per thread).
-// The exact FP32 integers become integers by adding 1.5 2^23 (full rate; the
-// conversion instruction is not); the biases this leaves are removed once at the end.
-// Where a launch has too few tiles for the SMs, ns CTAs take parts of a tile's K
-// range, add their 64-bit sums atomically (integers: any order gives the same value)
-// and the last one converts.
+// columns each), eight warps recombine the set of the group before in registers (64
+// 64-bit sums per thread).  Where a launch has too few tiles for the SMs, ns CTAs take
+// parts of a tile's K range, add their 64-bit sums atomically (integers: any order
+// gives the same value) and the last one converts.
 __global__ void __launch_bounds__(SL_THREADS, 1)
     k_syrk_sl(const __grid_constant__ CUtensorMap map_i, const __grid_constant__ CUtensorMap map_j, SlArgs A) {
   extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t full[SL_STAGES], empty[SL_STAGES], tfull[2], tempty[2], mma_done;
+  __shared__ __align__(8) SlBars bars;
   __shared__ uint32_t tmem_sh;
   __shared__ int last_sh;
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -411,137 +291,35 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
   const int kb0 = (int)((int64_t)A.nk * sp / A.ns), kb1 = (int)((int64_t)A.nk * (sp + 1) / A.ns);
   int64_t ti, tj;
   sl_tile(tile, A.t0, A.t1, &ti, &tj);
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < SL_STAGES; ++s) {
-      sl_init(&full[s], 1);
-      sl_init(&empty[s], 1);
-    }
-    for (int b = 0; b < 2; ++b) {
-      sl_init(&tfull[b], 1);
-      sl_init(&tempty[b], SL_EPI);
-    }
-    sl_init(&mma_done, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  }
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sl_u32(&tmem_sh)), "r"(512));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-  }
+  if (threadIdx.x == 0) sl_bars_init(&bars);
+  if (warp == 0) sl_tmem_alloc(&tmem_sh);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_sh;
   const int q = warp & 3, half = (warp - 2) >> 2;  // epilogue warp: TMEM lanes 32 q .., columns 16 half .. of a group
   const int row = q * 32 + lane;
-  const unsigned long long bias = ((unsigned long long)SL_MAGIC << 48) + ((257ull * SL_MAGIC) << 32) +
-                                  ((257ull * SL_MAGIC & 0xFFFFFFFFull) << 16) + (257ull * SL_MAGIC & 0xFFFFFFFFull);
 
   if (warp == 0 && lane == 0) {
-    for (int kb = kb0; kb < kb1; ++kb) {
-      const int w = kb - kb0, s = w % SL_STAGES;
-      if (!sl_wait(&empty[s], (uint32_t)((w / SL_STAGES) & 1) ^ 1u, A.status)) break;
-      uint8_t* st = smem + (size_t)s * SL_STAGE;
-      const int bi = (int)(ti * A.nk + kb), bj = (int)(tj * A.nk + kb);
-      sl_expect(&full[s], SL_STAGE);
-      sl_tma(&map_i, &full[s], st, 0, bi);
-      for (int j = 0; j < SL_NG; ++j) sl_tma(&map_j, &full[s], st + SL_BLOCK + j * SL_GROUP, j * SL_BN, bj);
-      if (kb + 2 < kb1) {
-        sl_prefetch(&map_i, 0, bi + 2);
-        if (ti != tj) sl_prefetch(&map_i, 0, bj + 2);
-      }
-    }
-  } else if (warp == 1 && lane == 0) {
-    for (int kb = kb0; kb < kb1; ++kb) {
-      const int w = kb - kb0, s = w % SL_STAGES;
-      if (!sl_wait(&full[s], (uint32_t)((w / SL_STAGES) & 1), A.status)) break;
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t base_i = sl_u32(smem + (size_t)s * SL_STAGE);
-      bool ok = true;
-#pragma unroll 1
-      for (int j = 0; j < SL_NG && ok; ++j) {
-        const int b = j & 1, use = 2 * w + (j >> 1);  // use-th filling of accumulator set b
-        ok = sl_wait(&tempty[b], (uint32_t)(use & 1) ^ 1u, A.status);
-        if (!ok) break;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t base_j = base_i + SL_BLOCK + j * SL_GROUP, dt = tmem + (uint32_t)(b * 256);
-#pragma unroll
-        for (int k = 0; k < SL_BK / 16; ++k)
-#pragma unroll
-          for (int t = 0; t < SL_S; ++t) {
-            // BF16 x BF16 -> FP32, K-major, M = 128, N = 32 (7 - t): digit t against the digits 0 .. 6 - t
-            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) |
-                                   ((uint32_t)((SL_BN * (SL_S - t)) >> 3) << 17) | ((uint32_t)(SL_BM >> 4) << 24);
-            const uint32_t acc = (k == 0 && t == 0) ? 0u : 1u;
-            asm volatile(
-                "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, "
-                "p;\n}\n" ::"r"(dt + (uint32_t)(t * SL_BN)),
-                "l"(sl_desc(base_i + t * SL_DIGIT + k * 32)), "l"(sl_desc(base_j + k * 32)), "r"(idesc), "r"(acc)
-                : "memory");
-          }
-        sl_commit(&tfull[b]);
-      }
-      if (!ok) break;
-      sl_commit(&empty[s]);
-    }
-    // every MMA of this CTA has completed before its TMEM is released
-    sl_commit(&mma_done);
-    for (uint32_t i = 0; i < SL_SPIN && !sl_try(&mma_done, 0u); ++i) {
-    }
+    int it = 0;
+    sl_produce<SL_NG>(&map_i, &map_j, smem, &bars, (int)(ti * A.nk) + kb0, (int)(tj * A.nk) + kb0, 0, kb1 - kb0, it, A.status);
+  } else if (warp == 1) {
+    int it = 0;
+    sl_issue<SL_NG, false>(smem, &bars, kb1 - kb0, it, A.status);
+    sl_issue_end(&bars, lane);
   } else if (warp >= 2) {
     unsigned long long acc[SL_NG][16];
 #pragma unroll
     for (int j = 0; j < SL_NG; ++j)
 #pragma unroll
       for (int c = 0; c < 16; ++c) acc[j][c] = 0ull;
-    int ok = 1;
-    const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * 16);
-    for (int kb = kb0; kb < kb1 && ok; ++kb) {
-#pragma unroll
-      for (int j = 0; j < SL_NG; ++j) {
-        if (ok) {  // (warp-uniform: the TMEM loads are warp-collective)
-          const int b = j & 1;
-          if (lane == 0) ok = sl_wait(&tfull[b], (uint32_t)(j >> 1), A.status);
-          ok = __shfl_sync(0xffffffffu, ok, 0);
-          __syncwarp();
-        }
-        if (ok) {
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            uint32_t r[SL_S][8];
-#pragma unroll
-            for (int g = 0; g < SL_S; ++g) sl_tmem_ld8(tbase + (uint32_t)((j & 1) * 256 + g * SL_BN + h * 8), r[g]);
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-            for (int g = 0; g < SL_S; ++g)
-#pragma unroll
-              for (int c = 0; c < 8; ++c) asm volatile("" : "+r"(r[g][c]));
-            if (h == 1) {  // the set's values are in registers
-              asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-              __syncwarp();
-              if (lane == 0) sl_arrive(&tempty[j & 1]);
-            }
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {
-              uint32_t v[SL_S];
-#pragma unroll
-              for (int g = 0; g < SL_S; ++g) v[g] = __float_as_uint(__uint_as_float(r[g][c]) + 12582912.0f);
-              // a_0 2^48 + (a_1 2^8 + a_2) 2^32 + (a_3 2^8 + a_4) 2^16 + (a_5 2^8 + a_6), biased
-              unsigned long long x = acc[j][h * 8 + c];
-              x += (unsigned long long)(v[3] * 256u + v[4]) * 65536ull;
-              x += (unsigned long long)(v[5] * 256u + v[6]);
-              x += (unsigned long long)(v[0] * 65536u + v[1] * 256u + v[2]) << 32;
-              acc[j][h * 8 + c] = x;
-            }
-          }
-        }
-      }
-    }
+    int it = 0;
+    sl_drain_init<false>(&bars, tmem, q, half, lane);
+    const bool ok = sl_drain<SL_NG, false>(acc, &bars, tmem, q, half, lane, kb1 - kb0, it, A.status);
     if (ok && *(volatile int*)A.status == 0) {
       if (A.ns == 1) {
-        const unsigned long long off = bias * (unsigned long long)(kb1 - kb0);
-        const int64_t gr = ti * SL_BM + row;
+        const unsigned long long off = SL_BIAS * (unsigned long long)(kb1 - kb0);
+        const int64_t gr = ti * SL_BM + sl_row<false>(q, lane, 0);
         if (gr < A.row1) {
           const int er = A.rexp[gr] - 62;
           double* p = A.out.at(gr, tj * SL_BM);
@@ -549,36 +327,33 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
           for (int j = 0; j < SL_NG; ++j)
 #pragma unroll
             for (int c = 0; c < 16; ++c) {
-              const int lc = j * SL_BN + half * 16 + c;
+              const int lc = sl_col<false>(half, lane, j, c);
               const int64_t gc = tj * SL_BM + lc;
               if (gc <= gr) p[lc] = scaled_to_double_rn((long long)(acc[j][c] - off), er + __ldg(A.rexp + gc));
             }
         }
       } else {
-        unsigned long long* p = A.part + (size_t)tile * (SL_BM * SL_BM) + row;
+        unsigned long long* p = A.part + (size_t)tile * (SL_BM * SL_BM);
 #pragma unroll
         for (int j = 0; j < SL_NG; ++j)
 #pragma unroll
           for (int c = 0; c < 16; ++c)
-            atomicAdd(p + (size_t)(j * SL_BN + half * 16 + c) * SL_BM, acc[j][c]);
+            atomicAdd(p + (size_t)sl_col<false>(half, lane, j, c) * SL_BM + sl_row<false>(q, lane, c), acc[j][c]);
       }
     }
   }
   __syncwarp();
-  // after an expired wait some copies may still be in flight: a bounded
-  // pause (~1 ms) lets them land before the CTA's shared memory is released
-  if (warp == 0 && lane == 0 && *(volatile int*)A.status != 0)
-    for (int i = 0; i < 1000; ++i) __nanosleep(1000);
+  if (warp == 0 && lane == 0) sl_pause(A.status);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   if (A.ns > 1) __threadfence();
   __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+  if (warp == 0) sl_tmem_free(tmem);
   if (A.ns > 1) {
     if (threadIdx.x == 0) last_sh = atomicAdd(A.ticket + tile, 1) == A.ns - 1;
     __syncthreads();
     if (last_sh && *(volatile int*)A.status == 0) {
       __threadfence();
-      const unsigned long long off = bias * (unsigned long long)A.nk;
+      const unsigned long long off = SL_BIAS * (unsigned long long)A.nk;
       const unsigned long long* p = A.part + (size_t)tile * (SL_BM * SL_BM);
       for (int e = threadIdx.x; e < SL_BM * SL_BM; e += SL_THREADS) {
         const int lr = e & (SL_BM - 1), lc = e >> 7;
@@ -606,7 +381,7 @@ size_t wl_sl_fixed_bytes(const cov_handle* h) {
          (size_t)SL_SPLIT_TILES * (SL_BM * SL_BM * 8 + sizeof(int));
 }
 
-static int sl_map(cov_handle* h, CUtensorMap* map, void* base, int64_t blocks, int box_rows) {
+int wl_sl_map(cov_handle* h, CUtensorMap* map, void* base, int64_t blocks, int box_rows) {
   auto fn = wl_encode_tiled();
   if (!fn) return wl_fail(h, COV_ERR_CUDA, "cuTensorMapEncodeTiled unavailable");
   cuuint64_t dims[4] = {SL_BK, SL_BM, SL_S, (cuuint64_t)blocks};
@@ -718,7 +493,7 @@ int wl_sl_syrk(cov_handle* h, bool tri, int nssc, OutMap out, int64_t row1, cuda
   CUtensorMap mi, mj;
   int rc;
   uint8_t* sl = tri ? h->Tsl : h->Asl;
-  if ((rc = sl_map(h, &mi, sl, nb * nk, SL_BM)) || (rc = sl_map(h, &mj, sl, nb * nk, SL_BN))) return rc;
+  if ((rc = wl_sl_map(h, &mi, sl, nb * nk, SL_BM)) || (rc = wl_sl_map(h, &mj, sl, nb * nk, SL_BN))) return rc;
   // CTAs per tile: with one per SM, the parts (of at least 16 K blocks) that finish in
   // the fewest waves of K blocks
   const int64_t sms = wl_num_sms();
@@ -744,10 +519,11 @@ int wl_sl_syrk(cov_handle* h, bool tri, int nssc, OutMap out, int64_t row1, cuda
   static std::once_flag attr_once[WL_MAX_DEVICES];
   static int attr_rc[WL_MAX_DEVICES];
   if (wl_once_per_device(attr_once, attr_rc, [] {
-        return (int)cudaFuncSetAttribute(k_syrk_sl, cudaFuncAttributeMaxDynamicSharedMemorySize, SL_SMEM);
+        return (int)cudaFuncSetAttribute(k_syrk_sl, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         SlShape<SL_NG>::kSmem);
       }) != 0)
     return wl_fail(h, COV_ERR_CUDA, "cudaFuncSetAttribute(k_syrk_sl) failed");
-  k_syrk_sl<<<(unsigned)(ntiles * ns), SL_THREADS, SL_SMEM, s>>>(mi, mj, a);
+  k_syrk_sl<<<(unsigned)(ntiles * ns), SL_THREADS, SlShape<SL_NG>::kSmem, s>>>(mi, mj, a);
   WL_LAUNCH(h, "k_syrk_sl");
   return COV_OK;
 }
