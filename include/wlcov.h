@@ -323,8 +323,9 @@ int cov_snr_noalloc(const double* d_C, int64_t ldc, const double* d_D, int64_t M
  * (Eq. CumulSN).  The eigenvalues of these covariances span ~23 decades, so
  * they come from one-sided Jacobi on the Cholesky factor, which keeps every
  * eigenvalue to high relative accuracy (in FP64, on the GPU): the factor of
- * cov_snr (FP64-accurate), then sweeps of plane rotations of column pairs of
- * L^T in round-robin order until a sweep rotates no pair (at most 60 sweeps).
+ * cov_snr (FP64-accurate) with the rows in order of descending variance, then
+ * sweeps of plane rotations of column pairs of L in round-robin order until a
+ * sweep rotates no pair (at most 60 sweeps).
  *
  * d_C: device, M x M FP64 with the lower triangle (the upper is not read),
  * leading dimension ldc >= M, rows in the handle's order; d_D: device, M.

@@ -199,7 +199,10 @@ static int selection(cov_handle* h, int slot, cudaStream_t s) {
   return COV_OK;
 }
 
-int wl_snr(cov_handle* h, const double* C, int64_t ldc, const double* D, int which, double* h_snr, cudaStream_t s) {
+// perm: another order of the selection's rows (the factor is then of that order, and the
+// prefix sums are of no use)
+int wl_snr(cov_handle* h, const double* C, int64_t ldc, const double* D, int which, double* h_snr, cudaStream_t s,
+           const int* perm) {
   int rc;
   if ((rc = selection(h, which, s))) return rc;
   const auto& z = h->sel[which];
@@ -226,7 +229,7 @@ int wl_snr(cov_handle* h, const double* C, int64_t ldc, const double* D, int whi
     h->allocated += sizeof(double) * need;
   }
   h->work_ld = ldw;
-  return factor_and_prefix(h, out_rows(h->work, ldw), Ms, z.perm, C, ldc, D, z.cnt, z.out, h_snr, s);
+  return factor_and_prefix(h, out_rows(h->work, ldw), Ms, perm ? perm : z.perm, C, ldc, D, z.cnt, z.out, h_snr, s);
 }
 
 // In place on the lower-packed tiles (rows in cumulative order)

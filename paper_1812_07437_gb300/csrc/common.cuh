@@ -290,7 +290,7 @@ int wl_snr_tiles(cov_handle* h, double* Ct, const double* D, double* h_snr, cuda
 int wl_assemble_band(cov_handle* h, int64_t row0, int64_t nrows, OutMap out, unsigned terms, int precision,
                      cudaStream_t s);
 int wl_snr(cov_handle* h, const double* d_C, int64_t ldc, const double* d_D, int which, double* h_snr,
-           cudaStream_t s);  // chol.cu
+           cudaStream_t s, const int* perm = nullptr);  // chol.cu
 int wl_gemm_lower_fp64(cov_handle* h, const double* A, int64_t lda, const double* B, int64_t ldb, double* C,
                        int64_t ldc, int64_t n, int64_t k, double alpha, double beta, bool lower_only,
                        cudaStream_t s);  // assemble.cu
