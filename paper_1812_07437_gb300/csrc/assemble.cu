@@ -615,11 +615,14 @@ static int prepare_operands(cov_handle* h, unsigned terms, int precision, cudaSt
   return COV_OK;
 }
 
-// Band assembly.  In the split form the band is cut into sub-bands of about
-// equal tile counts; the contraction of sub-band k+1 (main stream) runs while
-// the per-element products of sub-band k (side stream) are added, so the
-// gather's FP64 work and read-modify-write traffic hide under the tensor-core
-// kernel, which leaves most of each SM's issue slots and HBM bandwidth free.
+// Band assembly.  In the split form a large band is cut into up to eight sub-bands of
+// about equal tile counts; the contraction of sub-band k+1 (main stream) runs while the
+// per-element products of sub-band k (side stream) are added.  Every cut costs the
+// contraction part of a wave of tiles, and the products slow it while they run, for the
+// ~3% that the products take: M = 181350 (1655 waves) 1932 ms in eight against 1958 in
+// one; M = 24400 (30 waves) 35.1 against 31.7 + 1.4; M = 12944 (9 waves) 14.35 against
+// 9.0 + 0.5.  So a sub-band has at least BAND_WAVES waves.
+#define BAND_WAVES 64
 int wl_assemble_band(cov_handle* h, int64_t row0, int64_t nrows, OutMap out, unsigned terms, int precision,
                      cudaStream_t s) {
   int rc;
@@ -647,10 +650,10 @@ int wl_assemble_band(cov_handle* h, int64_t row0, int64_t nrows, OutMap out, uns
   };
   if (precision != COV_FP64 && (terms & COV_TERM_1H)) {
     const int nssc = (terms & COV_TERM_SSC) ? h->nchi : 0;
-    if ((rc = wl_side_stream(h))) return rc;
     // sub-band cuts at tile rows, about equal numbers of tiles each
     const int64_t ta = row0 / 256, tb = (row1 + 255) / 256;
-    const int nsub = (int)std::min<int64_t>(8, tb - ta);
+    const double waves = 0.5 * (double)(tb * (tb + 1) - ta * (ta + 1)) / wl_num_sms();
+    const int nsub = (int)std::max<int64_t>(1, std::min<int64_t>({8, tb - ta, (int64_t)(waves / BAND_WAVES)}));
     std::vector<int64_t> cut{row0};
     const double tot = 0.5 * (double)(tb * (tb + 1) - ta * (ta + 1));
     for (int k = 1; k < nsub; ++k) {
@@ -661,6 +664,18 @@ int wl_assemble_band(cov_handle* h, int64_t row0, int64_t nrows, OutMap out, uns
     }
     if (cut.back() != row1) cut.push_back(row1);
     if ((rc = wl_tc_status_reset(h, s))) return rc;
+    if (nsub == 1) {
+      int tk = wl_stage_begin(h, ST_SYRK_1H, s);
+      if ((rc = wl_syrk_tc_part(h, nssc, out, row0, row1, s))) return rc;
+      wl_stage_end(h, tk, s);
+      tk = wl_stage_begin(h, ST_GATHER, s);
+      gather(row0, row1, s);
+      WL_LAUNCH(h, "k_gather");
+      if ((rc = gauss(h, g, row0, row1, out, s))) return rc;
+      wl_stage_end(h, tk, s);
+      return wl_tc_status_check(h, s);
+    }
+    if ((rc = wl_side_stream(h))) return rc;
     WL_CHECK(h, cudaEventRecord(h->ev_panel, s));  // the side stream starts after the operands
     WL_CHECK(h, cudaStreamWaitEvent(h->side, h->ev_panel, 0));
     int tk = wl_stage_begin(h, ST_SYRK_1H, s);
