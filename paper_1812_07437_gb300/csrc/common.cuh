@@ -193,6 +193,7 @@ struct cov_handle {
   struct TileOrder {
     int kind = -1, group = 0;
     int64_t t0 = -1, t1 = -1, n = 0;
+    int64_t rest = 0, rest_tiles = 0;  // pair tiles of the last, partial wave, and their lower 128 x 128 tiles
     int2* p = nullptr;  // a slot of tile_ring
   } tile_cache[WL_TILE_CACHE];
   int2* tile_ring = nullptr;

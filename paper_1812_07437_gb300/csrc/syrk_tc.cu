@@ -318,6 +318,23 @@ __device__ __forceinline__ void umma_bf16(uint32_t dtmem, uint64_t ad, uint64_t 
       : "memory");
 }
 
+// The lane that issues a warp's MMAs and commits.  The issuing loop is run by the whole
+// warp, so that addresses and descriptors stay in uniform registers (inside a one-lane
+// branch every operand is moved there first).
+__device__ __forceinline__ uint32_t elect_lane() {
+  uint32_t leader;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(leader));
+  return leader;
+}
+__device__ __forceinline__ void umma_bf16_elected(uint32_t dtmem, uint64_t ad, uint64_t bd, uint32_t idesc,
+                                                  uint32_t acc, uint32_t leader) {
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n @q "
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtmem),
+      "l"(ad), "l"(bd), "r"(idesc), "r"(acc), "r"(leader)
+      : "memory");
+}
+
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                : "memory");
@@ -606,11 +623,11 @@ __device__ __forceinline__ void tma_load_2d_pair(const CUtensorMap* map, uint32_
       : "memory");
 }
 __device__ __forceinline__ void umma_bf16_pair(uint32_t dtmem, uint64_t ad, uint64_t bd, uint32_t idesc,
-                                               uint32_t acc) {
+                                               uint32_t acc, uint32_t leader) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
-          dtmem),
-      "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
+      "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n @q "
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtmem),
+      "l"(ad), "l"(bd), "r"(idesc), "r"(acc), "r"(leader)
       : "memory");
 }
 // arrive on one barrier (of either CTA) when the pair MMAs issued so far complete
@@ -633,7 +650,7 @@ __device__ __forceinline__ uint32_t idesc_bf16_256x256() {
 // r_base .. r_base + 127 and the nh column halves of 256 from col0, staged
 // through shared memory (transpose) as in tile_epilogue.
 __device__ __forceinline__ void pair_epilogue(uint8_t* smem, uint32_t tmem, int warp, int lane, int64_t r_base,
-                                              int64_t col0, int nh, int64_t M, const double* __restrict__ rscale,
+                                              int64_t col0, int nc, int64_t M, const double* __restrict__ rscale,
                                               const OutMap& out) {
   uint32_t* stg = (uint32_t*)smem + warp * (32 * 33 + 32);
   int* erow = (int*)(stg + 32 * 33);
@@ -641,23 +658,20 @@ __device__ __forceinline__ void pair_epilogue(uint8_t* smem, uint32_t tmem, int 
   const int64_t gi = r0 + lane;
   erow[lane] = (gi < M) ? pow2_exp(rscale[gi]) : 0;
 #pragma unroll 1
-  for (int h = 0; h < nh; ++h) {
-#pragma unroll 1
-    for (int c = 0; c < 8; ++c) {
-      float v[32];
-      tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(256 * h + c * 32), v);
+  for (int c = 0; c < nc; ++c) {  // 32 columns at a time
+    float v[32];
+    tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(c * 32), v);
 #pragma unroll
-      for (int jj = 0; jj < 32; ++jj) stg[lane * 33 + jj] = __float_as_uint(v[jj]);
-      __syncwarp();
-      const int64_t gj = col0 + 256 * h + c * 32 + lane;
-      const int ej = (gj < M) ? pow2_exp(rscale[gj]) : 0;
+    for (int jj = 0; jj < 32; ++jj) stg[lane * 33 + jj] = __float_as_uint(v[jj]);
+    __syncwarp();
+    const int64_t gj = col0 + c * 32 + lane;
+    const int ej = (gj < M) ? pow2_exp(rscale[gj]) : 0;
 #pragma unroll 4
-      for (int rr = 0; rr < 32; ++rr) {
-        const int64_t gr = r0 + rr;
-        if (gr < M && gj < M && gj <= gr) *out.at(gr, gj) = f32_scaled(stg[rr * 33 + lane], erow[rr] + ej);
-      }
-      __syncwarp();
+    for (int rr = 0; rr < 32; ++rr) {
+      const int64_t gr = r0 + rr;
+      if (gr < M && gj < M && gj <= gr) *out.at(gr, gj) = f32_scaled(stg[rr * 33 + lane], erow[rr] + ej);
     }
+    __syncwarp();
   }
 }
 
@@ -770,13 +784,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128, 1)
       const uint32_t ph = (uint32_t)(kb / PR_STAGES) & 1u;
       if (!mbar_wait(&empty_bar[st], ph ^ 1u, &abort_flag, status)) break;
     }
-  } else if (warp == 1 && lane == 0 && p == 0) {
+  } else if (warp == 1 && p == 0) {
+    const uint32_t leader = elect_lane();
     const uint32_t idesc = idesc_bf16_256x256();
     const uint32_t empty_peer0 = cluster_addr(&empty_bar[0], 1), acc_peer = cluster_addr(&acc_bar, 1);
     for (int kb = 0; kb < nk; ++kb) {
       const int st = kb % PR_STAGES;
       const uint32_t ph = (uint32_t)(kb / PR_STAGES) & 1u;
-      if (!mbar_wait(&full_bar[st], ph, &abort_flag, status)) break;
+      if (!__all_sync(0xffffffffu, mbar_wait(&full_bar[st], ph, &abort_flag, status))) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t sa = smem_u32(smem + (size_t)st * PR_STAGE_BYTES);
       const uint32_t a_hi = sa, a_lo = sa + PR_HALF;
@@ -789,22 +804,27 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128, 1)
         for (int k = 0; k < TW_BK / 16; ++k) {
           const uint32_t o = k * 32;
           const uint32_t first = (kb == 0 && k == 0) ? 0u : 1u;
-          umma_bf16_pair(dt, umma_desc_sw64(a_hi + o), umma_desc_sw64(b_hi + o), idesc, first);
-          umma_bf16_pair(dt, umma_desc_sw64(a_hi + o), umma_desc_sw64(b_lo + o), idesc, 1u);
-          umma_bf16_pair(dt, umma_desc_sw64(a_lo + o), umma_desc_sw64(b_hi + o), idesc, 1u);
+          umma_bf16_pair(dt, umma_desc_sw64(a_hi + o), umma_desc_sw64(b_hi + o), idesc, first, leader);
+          umma_bf16_pair(dt, umma_desc_sw64(a_hi + o), umma_desc_sw64(b_lo + o), idesc, 1u, leader);
+          umma_bf16_pair(dt, umma_desc_sw64(a_lo + o), umma_desc_sw64(b_hi + o), idesc, 1u, leader);
         }
       }
-      umma_commit_pair(smem_u32(&empty_bar[st]));
-      umma_commit_pair(empty_peer0 + 8u * (uint32_t)st);
+      if (leader) {
+        umma_commit_pair(smem_u32(&empty_bar[st]));
+        umma_commit_pair(empty_peer0 + 8u * (uint32_t)st);
+      }
+      __syncwarp();
     }
-    umma_commit_pair(smem_u32(&acc_bar));
-    umma_commit_pair(acc_peer);
+    if (leader) {
+      umma_commit_pair(smem_u32(&acc_bar));
+      umma_commit_pair(acc_peer);
+    }
   }
   __syncwarp();
   const bool have = mbar_wait(&acc_bar, 0u, &abort_flag, status);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (have && !abort_flag && *(volatile int*)status == 0)
-    pair_epilogue(smem, tmem, warp, lane, (int64_t)row_i + 128 * p, row_j, two ? 2 : 1, M, rscale, out);
+    pair_epilogue(smem, tmem, warp, lane, (int64_t)row_i + 128 * p, row_j, two ? 16 : 8, M, rscale, out);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   cluster_sync_all();  // both CTAs are past their MMAs, copies and epilogues
@@ -819,6 +839,124 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128, 1)
   }
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
   cluster_sync_all();  // no CTA leaves while its peer may still reach it
+}
+
+// ---------------------------------------------------------------- 128 x 128 tiles
+// The last, partial wave of pair tiles (and all of a small matrix): a 256 x 512 pair tile
+// takes as long for one column as for 512, and a wave of r < 76 pairs leaves the other
+// SMs idle.  Its lower 128 x 128 tiles go to one CTA each, the same K blocks and products
+// in the same order (the same sums bit for bit).  Bound by L2 where all SMs take part
+// (32 KB per K block and tile against 480 cycles of MMAs), by the MMAs and the latency of
+// a K block where few do.  A tile on the diagonal has its columns in its rows' panel; one
+// at the right edge multiplies its columns rounded up to 16 only.
+//
+// A wave of pair tiles of K = 32768 takes 0.90 ms, one of these tiles ~0.33: the rest goes
+// this way while it is at most two waves of them (42 pairs, 300 tiles: 0.90 -> 0.67 ms;
+// 49 pairs, 351 tiles: 0.90 and 0.905).  M = 51, K = 4160: contraction 86 -> 35 us;
+// M = 1830, K = 12288: 0.364 -> 0.120 ms; M = 6375 (17 of 169 pairs): 1.12 -> 1.01 ms.
+#define SB_MAX_WAVES 2
+#define SB_STAGES 6
+#define SB_STAGE_BYTES (4 * PR_HALF)  // A hi/lo, B hi/lo
+#define SB_SMEM (SB_STAGES * SB_STAGE_BYTES + 1024)
+
+__global__ void __launch_bounds__(128, 1)
+    k_syrk_sub(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo, int64_t M,
+               int nk, const double* __restrict__ rscale, OutMap out, int* status, const int2* __restrict__ pairs) {
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ __align__(8) uint64_t full_bar[SB_STAGES];
+  __shared__ __align__(8) uint64_t empty_bar[SB_STAGES];
+  __shared__ __align__(8) uint64_t acc_bar;
+  __shared__ uint32_t tmem_base_sh;
+  __shared__ volatile int abort_flag;
+
+  const int2 pt = pairs[blockIdx.x >> 3];
+  const int64_t ti = pt.x, tj = pt.y;
+  if (tj < 0 || tj > ti || ti * TW_BM >= M) {  // outside the lower triangle: reported, skipped
+    if (threadIdx.x == 0) atomicExch(status, 2);
+    return;
+  }
+  const int64_t row0 = ti * TW_BM + 128 * (blockIdx.x & 1), col0 = tj * TW_BM + 128 * ((blockIdx.x >> 1) & 3);
+  if (row0 >= M || col0 > row0) return;
+  const bool diag = row0 == col0;
+  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+  if (threadIdx.x == 0) {
+    abort_flag = 0;
+    for (int s = 0; s < SB_STAGES; ++s) {
+      mbar_init(&full_bar[s], 1);
+      mbar_init(&empty_bar[s], 1);
+    }
+    mbar_init(&acc_bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_sh)),
+                 "r"(128));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = tmem_base_sh;
+  const int cols = (int)(M - col0 < 128 ? M - col0 : 128);
+
+  if (warp == 0 && lane == 0) {
+    const int64_t yi0 = (row0 >> 8) * nk * TW_BM + (row0 & 255), yj0 = (col0 >> 8) * nk * TW_BM + (col0 & 255);
+    int issued = 0;
+    for (int kb = 0; kb < nk; ++kb) {
+      const int s = kb % SB_STAGES;
+      if (!mbar_wait(&empty_bar[s], ((uint32_t)(kb / SB_STAGES) & 1u) ^ 1u, &abort_flag, status)) break;
+      issued = kb + 1;
+      uint8_t* st = smem + (size_t)s * SB_STAGE_BYTES;
+      mbar_expect_tx(&full_bar[s], (diag ? 2 : 4) * PR_HALF);
+      const int yi = (int)(yi0 + (int64_t)kb * TW_BM), yj = (int)(yj0 + (int64_t)kb * TW_BM);
+      tma_load_2d(&map_hi, &full_bar[s], st, 0, yi);
+      tma_load_2d(&map_lo, &full_bar[s], st + PR_HALF, 0, yi);
+      if (!diag) {
+        tma_load_2d(&map_hi, &full_bar[s], st + 2 * PR_HALF, 0, yj);
+        tma_load_2d(&map_lo, &full_bar[s], st + 3 * PR_HALF, 0, yj);
+      }
+    }
+    if (abort_flag) {
+      for (int kb = issued - SB_STAGES < 0 ? 0 : issued - SB_STAGES; kb < issued; ++kb)
+        for (uint32_t i = 0; i < TC_SPIN_LIMIT && !mbar_try(&full_bar[kb % SB_STAGES], (uint32_t)(kb / SB_STAGES) & 1u); ++i) {
+        }
+    }
+  } else if (warp == 1) {
+    const uint32_t leader = elect_lane();
+    // kind::f16, BF16 x BF16 -> FP32, K-major, M = 128
+    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)((cols + 15) / 16 * 2) << 17) | (8u << 24);
+    const uint32_t boff = diag ? 0u : 2u * PR_HALF;
+    for (int kb = 0; kb < nk; ++kb) {
+      const int s = kb % SB_STAGES;
+      if (!__all_sync(0xffffffffu,
+                      mbar_wait(&full_bar[s], (uint32_t)(kb / SB_STAGES) & 1u, &abort_flag, status)))
+        break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t a_hi = smem_u32(smem + (size_t)s * SB_STAGE_BYTES), a_lo = a_hi + PR_HALF;
+      const uint32_t b_hi = a_hi + boff, b_lo = b_hi + PR_HALF;
+#pragma unroll
+      for (int k = 0; k < TW_BK / 16; ++k) {
+        const uint32_t o = k * 32;
+        umma_bf16_elected(tmem, umma_desc_sw64(a_hi + o), umma_desc_sw64(b_hi + o), idesc, kb == 0 && k == 0 ? 0u : 1u,
+                          leader);
+        umma_bf16_elected(tmem, umma_desc_sw64(a_hi + o), umma_desc_sw64(b_lo + o), idesc, 1u, leader);
+        umma_bf16_elected(tmem, umma_desc_sw64(a_lo + o), umma_desc_sw64(b_hi + o), idesc, 1u, leader);
+      }
+      if (leader) umma_commit(&empty_bar[s]);
+      __syncwarp();
+    }
+    if (leader) umma_commit(&acc_bar);
+  }
+  __syncwarp();
+  const bool have = mbar_wait(&acc_bar, 0u, &abort_flag, status);
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if (have && !abort_flag) pair_epilogue(smem, tmem, warp, lane, row0, col0, (cols + 31) / 32, M, rscale, out);
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(128));
 }
 
 // ---------------------------------------------------------------- host side
@@ -942,12 +1080,15 @@ int wl_trows_split(cov_handle* h, cudaStream_t s) {
 // (ti, tj), tj <= ti, of tile rows [t0, t1), row by row.  kind 1: the pair
 // tiles (ti, tj), tj even, each covering the lower tiles (ti, tj) and
 // (ti, tj + 1) (the second only when tj + 1 <= ti).
-int wl_tile_order(cov_handle* h, int kind, int64_t t0, int64_t t1, const int2** tiles, int64_t* n, cudaStream_t s) {
+// (declared here: the launch orders need the width of a wave)
+static int pair_clusters_ok();
+
+static int wl_tile_order(cov_handle* h, int kind, int64_t t0, int64_t t1, const cov_handle::TileOrder** order,
+                         cudaStream_t s) {
   const int group = kind == 1 ? h->pr_group : 0;
   for (auto& c : h->tile_cache)
     if (c.p && c.kind == kind && c.group == group && c.t0 == t0 && c.t1 == t1) {
-      *tiles = c.p;
-      *n = c.n;
+      *order = &c;
       return COV_OK;
     }
   std::vector<int2> v;
@@ -999,8 +1140,11 @@ int wl_tile_order(cov_handle* h, int kind, int64_t t0, int64_t t1, const int2** 
   c.t0 = t0;
   c.t1 = t1;
   c.n = (int64_t)v.size();
-  *tiles = c.p;
-  *n = c.n;
+  c.rest = kind == 1 ? c.n % pair_clusters_ok() : 0;
+  c.rest_tiles = 0;
+  for (size_t e = v.size() - (size_t)c.rest; e < v.size(); ++e)  // columns 2 y .. 2 y + 3 against rows 2 x, 2 x + 1
+    for (int r = 2 * v[e].x; r < 2 * v[e].x + 2; ++r) c.rest_tiles += std::min(4, r - 2 * v[e].y + 1);
+  *order = &c;
   return COV_OK;
 }
 
@@ -1037,16 +1181,29 @@ static int launch_tc(cov_handle* h, const void* hi, const void* lo, const double
   if (row1 < 0 || row1 > rows) row1 = rows;
   int64_t t0 = r0 / TW_BM, t1 = (row1 + TW_BM - 1) / TW_BM;
   if (t1 <= t0) return COV_OK;
-  const int2* tiles = nullptr;
-  int64_t nblk = 0;
+  const cov_handle::TileOrder* o = nullptr;
   if (h->tc_kernel != 0 && pair_clusters_ok()) {
     CUtensorMap mhi, mlo;
     if ((rc = make_map(h, &mhi, (void*)hi, rows, Kp, 128))) return rc;
     if ((rc = make_map(h, &mlo, (void*)lo, rows, Kp, 128))) return rc;
-    if ((rc = wl_tile_order(h, 1, t0, t1, &tiles, &nblk, s))) return rc;
-    k_syrk_pair<<<(unsigned)(2 * nblk), 128, PR_SMEM, s>>>(mhi, mlo, rows, Kp / TW_BK, rscale, out, h->tc_status,
-                                                           tiles);
-    WL_LAUNCH(h, "k_syrk_pair");
+    if ((rc = wl_tile_order(h, 1, t0, t1, &o, s))) return rc;
+    static std::once_flag sub_once[WL_MAX_DEVICES];
+    static int sub_rc[WL_MAX_DEVICES];
+    if (wl_once_per_device(sub_once, sub_rc, [] {
+          return (int)cudaFuncSetAttribute(k_syrk_sub, cudaFuncAttributeMaxDynamicSharedMemorySize, SB_SMEM);
+        }) != 0)
+      return wl_fail(h, COV_ERR_CUDA, "cudaFuncSetAttribute(k_syrk_sub) failed");
+    const int64_t sub = o->rest_tiles <= SB_MAX_WAVES * wl_num_sms() ? o->rest : 0, whole = o->n - sub;
+    if (whole) {
+      k_syrk_pair<<<(unsigned)(2 * whole), 128, PR_SMEM, s>>>(mhi, mlo, rows, Kp / TW_BK, rscale, out, h->tc_status,
+                                                              o->p);
+      WL_LAUNCH(h, "k_syrk_pair");
+    }
+    if (sub) {
+      k_syrk_sub<<<(unsigned)(8 * sub), 128, SB_SMEM, s>>>(mhi, mlo, rows, Kp / TW_BK, rscale, out, h->tc_status,
+                                                           o->p + whole);
+      WL_LAUNCH(h, "k_syrk_sub");
+    }
   } else {
     CUtensorMap mhi, mlo;
     if ((rc = make_map(h, &mhi, (void*)hi, rows, Kp))) return rc;
@@ -1057,8 +1214,8 @@ static int launch_tc(cov_handle* h, const void* hi, const void* lo, const double
           return (int)cudaFuncSetAttribute(k_syrk_tc256, cudaFuncAttributeMaxDynamicSharedMemorySize, TW_SMEM);
         }) != 0)
       return wl_fail(h, COV_ERR_CUDA, "cudaFuncSetAttribute(k_syrk_tc256) failed");
-    if ((rc = wl_tile_order(h, 0, t0, t1, &tiles, &nblk, s))) return rc;
-    k_syrk_tc256<<<(unsigned)nblk, 128, TW_SMEM, s>>>(mhi, mlo, rows, Kp / TW_BK, rscale, out, h->tc_status, tiles);
+    if ((rc = wl_tile_order(h, 0, t0, t1, &o, s))) return rc;
+    k_syrk_tc256<<<(unsigned)o->n, 128, TW_SMEM, s>>>(mhi, mlo, rows, Kp / TW_BK, rscale, out, h->tc_status, o->p);
     WL_LAUNCH(h, "k_syrk_tc256");
   }
   return COV_OK;
