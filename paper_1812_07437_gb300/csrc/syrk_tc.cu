@@ -62,206 +62,256 @@ __global__ void k_rows_prep(int nchi, int nm, double inv_omega, const cov_cosmol
 // Rows that share their ell bins share the (n, q) part of the 1-halo factor:
 // a P row of bin b has F_b[n][q] = g2[n][q] c2[n] U_b[n][q]^2, a B row of
 // triangle (a, b, c) has F_abc[n][q] = g3[n][q] c3[n] U_a U_b U_c, and the row
-// itself is F[n][q] times the product of its lensing kernels W_i(chi_n).  One
-// block per (signature s, node n) stores F[s][n][.] / 2^E[s][n] in FP32 (its
-// largest magnitude in [0.5, 1)), E[s][n] and the FP64 maximum.
-// pairs: signatures are the bin pairs b1 <= b2 (trispectrum rows, mu = 2)
-// instead of the P bins and B triangles.
-__global__ void k_rows_sig(int nl, int ntri, int nchi, int nm, const int32_t* tris, const double* U, const double* g2,
-                           const double* g3, const double* c2, const double* c3, float* F, int* E, double* Mx,
-                           int pairs) {
-  __shared__ double red[32];
-  int s = blockIdx.x, n = blockIdx.y;
-  bool isP = pairs || s < nl;
-  int a, b, c;
+// itself is F[n][q] times the product of its lensing kernels W_i(chi_n).  A
+// warp takes `per` signatures of one node and stores for each F[s][n][.] /
+// 2^E[s][n] in FP32 (its largest magnitude in [0.5, 1)), E[s][n] and the FP64
+// maximum.  pairs: signatures are the bin pairs b1 <= b2 (trispectrum rows,
+// mu = 2) instead of the P bins and B triangles.
+//
+// Bound by FP64 multiplications (a warp's takes 64 cycles): neighbouring
+// signatures differ in the last bin, so the product of the others stays in
+// registers, the maximum is an integer one, and the scaled FP32 value is formed from the bits.
+// 657 signatures of 256 x 128: 463 -> 183 us (one block per signature and
+// node, every value computed twice).
+// RN(v 2^-e) in FP32, by integer operations where the result is a normal number below 2
+// (an FP64 conversion takes as long as a multiplication)
+__device__ __forceinline__ float f32_shifted(double v, int e) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const int E = (int)((b >> 52) & 0x7FFu) - 896 - e;  // FP32 exponent field
+  if (E <= 0 || E > 127) return (float)ldexp(v, -e);
+  const unsigned m = (unsigned)((b + 0x0FFFFFFFull + ((b >> 29) & 1ull)) >> 29) & 0x7FFFFFu;
+  // a mantissa that rounds up to 2 carries into the exponent
+  const unsigned carry = (m == 0u && (b & 0x000FFFFFFFFFFFFFull) != 0ull && ((b >> 29) & 0x7FFFFFull) == 0x7FFFFFull);
+  return __uint_as_float((unsigned)(b >> 63) << 31 | ((unsigned)E + carry) << 23 | m);
+}
+
+__global__ void __launch_bounds__(256)
+    k_rows_sig(int nl, int nsig, int nchi, int nm, int per, const int32_t* __restrict__ tris,
+               const double* __restrict__ U, const double* __restrict__ g2, const double* __restrict__ g3,
+               const double* __restrict__ c2, const double* __restrict__ c3, float* F, int* E, double* Mx, int pairs) {
+  const int lane = threadIdx.x & 31, n = blockIdx.y;
+  const int s0 = (blockIdx.x * 8 + (threadIdx.x >> 5)) * per, s1 = min(nsig, s0 + per);
+  if (s0 >= nsig) return;
+  const size_t K = (size_t)nchi * nm;
+  const double* Un = U + (size_t)n * nm;
+  int a = 0, b = 0, c = 0, la = -1, lb = -1, lp = -1;
   if (pairs) {
-    a = 0;
     int base = 0;
-    while (base + (nl - a) <= s) {
+    while (base + (nl - a) <= s0) {
       base += nl - a;
       ++a;
     }
-    b = a + (s - base);
-    c = b;
-  } else if (isP) {
-    a = b = c = s;
-  } else {
-    a = tris[3 * (s - nl)];
-    b = tris[3 * (s - nl) + 1];
-    c = tris[3 * (s - nl) + 2];
+    b = a + (s0 - base) - 1;
   }
-  const size_t K = (size_t)nchi * nm;
-  const double* Ua = U + a * K + (size_t)n * nm;
-  const double* Ub = U + b * K + (size_t)n * nm;
-  const double* Uc = U + c * K + (size_t)n * nm;
-  const double* g = (isP ? g2 : g3) + (size_t)n * nm;
-  double cn = isP ? c2[n] : c3[n];
-  auto value = [&](int q) { return isP ? g[q] * cn * Ua[q] * Ub[q] : g[q] * cn * Ua[q] * Ub[q] * Uc[q]; };
-  double mx = 0.0;
-  for (int q = threadIdx.x; q < nm; q += blockDim.x) mx = fmax(mx, fabs(value(q)));
-  mx = warp_max(mx);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double t = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
-    t = warp_max(t);
-    if (threadIdx.x == 0) red[0] = t;
-  }
-  __syncthreads();
-  mx = red[0];
-  int e = 0;
-  if (mx > 0.0) frexp(mx, &e);
-  float* Fo = F + (size_t)s * K + (size_t)n * nm;
-  for (int q = threadIdx.x; q < nm; q += blockDim.x) Fo[q] = (float)ldexp(value(q), -e);
-  if (threadIdx.x == 0) {
-    E[(size_t)s * nchi + n] = e;
-    Mx[(size_t)s * nchi + n] = mx;
-  }
-}
-
-// One block per row a: entries 0..K-1 are the 1-halo factor row; when
-// nssc > 0, entries K..K+nssc-1 are the super-sample row S[a][n] (so that one
-// contraction gives A A^T + S S^T); the rest of Kp is zero.  The row is scaled
-// by an exact power of two s_a (largest entry in [0.5, 1)) and split into
-// BF16 hi/lo.  FP64 work is per node (kernel products, row maximum, the
-// super-sample entries); each factor entry is one FP32 product of the
-// signature table and a per-node FP32 weight, exact to a few 2^-24, well
-// inside the 2^-17 of the hi/lo split.
-__global__ void k_rows_split(int64_t M, int nl, int nchi, int nm, int Kp, int nssc, const int32_t* rd,
-                             const double* W, const float* F, const int* E, const double* Mx, const double* wchi,
-                             const double* sigw2, const double* chi, const double* RP3, const double* RB3,
-                             __nv_bfloat16* hi, __nv_bfloat16* lo, double* rscale) {
-  extern __shared__ double rs_sh[];  // [nchi] node weights, [nchi] super-sample entries
-  __shared__ double red[32];
-  int64_t a = blockIdx.x;
-  if (a >= M) return;
-  const int32_t* r = rd + 8 * a;
-  const int K = nchi * nm;
-  const bool isP = (r[0] == 0);
-  const int sg = isP ? r[1] : nl + r[7];
-  const double* W1 = W + r[4] * nchi;
-  const double* W2 = W + r[5] * nchi;
-  const double* W3 = W + (isP ? r[4] : r[6]) * nchi;
-  const int* Es = E + (size_t)sg * nchi;
-  const double* Ms = Mx + (size_t)sg * nchi;
-  double* wsh = rs_sh;
-  double* ssh = rs_sh + nchi;
-  // pass 1 (per node): kernel products, super-sample entries, row maximum
-  double mx = 0.0;
-  for (int n = threadIdx.x; n < nchi; n += blockDim.x) {
-    double w = W1[n] * W2[n];
-    if (!isP) w *= W3[n];
-    wsh[n] = w;
-    mx = fmax(mx, fabs(w) * Ms[n]);
-    double v = 0.0;
-    if (n < nssc) {
-      double ch = chi[n], c2_ = ch * ch;
-      v = sqrt(wchi[n] * sigw2[n]) * w;
-      v = isP ? v / c2_ * RP3[r[1] * nchi + n] : v / (c2_ * c2_) * RB3[r[7] * nchi + n];
-      mx = fmax(mx, fabs(v));
+  double head[4];  // g c_mu U_a (P, pairs) or g c_mu U_a U_b (B) of the lane's first four entries
+  for (int s = s0; s < s1; ++s) {
+    const bool isP = pairs || s < nl;
+    if (pairs) {
+      if (++b == nl) b = ++a;
+    } else if (isP) {
+      a = b = s;
+    } else {
+      a = tris[3 * (s - nl)];
+      b = tris[3 * (s - nl) + 1];
+      c = tris[3 * (s - nl) + 2];
     }
-    ssh[n] = v;
+    const double* g = (isP ? g2 : g3) + (size_t)n * nm;
+    const double cn = isP ? c2[n] : c3[n];
+    const double* Ul = Un + (size_t)(isP ? b : c) * K;
+    auto front = [&](int q) {
+      const double v = g[q] * cn * Un[a * K + q];
+      return isP ? v : v * Un[b * K + q];
+    };
+    if (a != la || (!isP && b != lb) || (int)isP != lp) {
+      la = a;
+      lb = b;
+      lp = (int)isP;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) head[k] = lane + 32 * k < nm ? front(lane + 32 * k) : 0.0;
+    }
+    double v[4];
+    unsigned long long mb = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int q = lane + 32 * k;
+      v[k] = q < nm ? head[k] * Ul[q] : 0.0;
+      const unsigned long long w = (unsigned long long)__double_as_longlong(v[k]) & 0x7FFFFFFFFFFFFFFFull;
+      mb = w > mb ? w : mb;
+    }
+    for (int q = lane + 128; q < nm; q += 32) {
+      const unsigned long long w =
+          (unsigned long long)__double_as_longlong(front(q) * Ul[q]) & 0x7FFFFFFFFFFFFFFFull;
+      mb = w > mb ? w : mb;
+    }
+    const unsigned hi = __reduce_max_sync(~0u, (unsigned)(mb >> 32));
+    const unsigned lo = __reduce_max_sync(~0u, (unsigned)(mb >> 32) == hi ? (unsigned)mb : 0u);
+    const double mx = __hiloint2double((int)hi, (int)lo);
+    int e = 0;
+    if (mx > 0.0) frexp(mx, &e);
+    float* Fo = F + (size_t)s * K + (size_t)n * nm;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int q = lane + 32 * k;
+      if (q < nm) Fo[q] = f32_shifted(v[k], e);
+    }
+    for (int q = lane + 128; q < nm; q += 32) Fo[q] = f32_shifted(front(q) * Ul[q], e);
+    if (lane == 0) {
+      E[(size_t)s * nchi + n] = e;
+      Mx[(size_t)s * nchi + n] = mx;
+    }
   }
-  mx = warp_max(mx);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double t = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
-    t = warp_max(t);
-    if (threadIdx.x == 0) red[0] = t;
-  }
-  __syncthreads();
-  mx = red[0];
-  int ex = 0;
-  if (mx > 0.0) frexp(mx, &ex);
-  // pass 2 (per node): FP32 weights relative to the row scale 2^ex
-  float* wf = (float*)(rs_sh + 2 * nchi);
-  float* sf = wf + nchi;
-  for (int n = threadIdx.x; n < nchi; n += blockDim.x) {
-    wf[n] = (float)ldexp(wsh[n], Es[n] - ex);
-    sf[n] = (float)ldexp(ssh[n], -ex);
-  }
-  __syncthreads();
-  // pass 3 (per entry pair): one FP32 product, BF16 hi/lo split, paired stores
-  const float* Fs = F + (size_t)sg * K;
-  const int Kt = K + nssc;
-  const int nk = Kp / TW_BK;
-  auto value = [&](int kk) -> float {
-    if (kk < K) return Fs[kk] * wf[(unsigned)kk / (unsigned)nm];
-    return kk < Kt ? sf[kk - K] : 0.0f;
-  };
-  for (int kk = 2 * threadIdx.x; kk < Kp; kk += 2 * blockDim.x) {
-    float x0 = value(kk), x1 = value(kk + 1);
-    __nv_bfloat162 h2 = __floats2bfloat162_rn(x0, x1);
-    __nv_bfloat162 l2 = __floats2bfloat162_rn(x0 - __low2float(h2), x1 - __high2float(h2));
-    int64_t o = blk_off(a, kk, nk);
-    *(__nv_bfloat162*)(hi + o) = h2;
-    *(__nv_bfloat162*)(lo + o) = l2;
-  }
-  if (threadIdx.x == 0) rscale[a] = ldexp(1.0, ex);
 }
 
-// Trispectrum rows of the PT term, one block per leg pair (L1 <= L2),
-// L = bin * n_t + tomo: T[(n, q)] = sqrt(w_n omega_q f_nq) (m_q/rho)^2
-// chi_n^-3 W_t1 W_t2 U_b1 U_b2, i.e. the pair signature (b1, b2) times the
-// node weight sqrt(Omega) W_t1(chi_n) W_t2(chi_n); scaled and split as
-// k_rows_split does.
-__global__ void k_trows_split(int64_t ntrow, int nleg, int nt, int nl, int nchi, int nm, int Kp, double sqrt_omega,
-                              const double* W, const float* F, const int* E, const double* Mx, __nv_bfloat16* hi,
-                              __nv_bfloat16* lo, double* rscale) {
-  extern __shared__ double ts_sh[];  // [nchi] node weights (FP64), then [nchi] FP32
-  __shared__ double red[32];
-  int64_t r = blockIdx.x;
-  if (r >= ntrow) return;
-  int L1 = 0;
-  int64_t base = 0;
-  while (base + (nleg - L1) <= r) {
-    base += nleg - L1;
-    ++L1;
+// Signatures per warp: enough warps to fill the device first
+static int sig_per_warp(int nsig, int nchi) {
+  return (int)std::max<int64_t>(1, std::min<int64_t>(16, (int64_t)nsig * nchi / (32 * wl_num_sms())));
+}
+
+// Factor rows.  TRI false: row a of the data vector; entries 0..K-1 are the
+// 1-halo factor row; when nssc > 0, entries K..K+nssc-1 are the super-sample
+// row S[a][n] (so that one contraction gives A A^T + S S^T); the rest of Kp is
+// zero.  TRI true: the trispectrum row of leg pair r (L1 <= L2, L = bin * n_t +
+// tomo), T[(n, q)] = sqrt(w_n omega_q f_nq) (m_q/rho)^2 chi_n^-3 W_t1 W_t2 U_b1
+// U_b2, i.e. the pair signature (b1, b2) times the node weight sqrt(Omega)
+// W_t1(chi_n) W_t2(chi_n).  The row is scaled by an exact power of two (largest
+// entry in [0.5, 1)) and split into BF16 hi/lo.  FP64 work is per node (kernel
+// products, row maximum, the super-sample entries); each factor entry is one
+// FP32 product of the signature table and a per-node FP32 weight, exact to a few
+// 2^-24, well inside the 2^-17 of the hi/lo split.
+//
+// A block takes every gridDim-th row, so that the square roots and divides of the
+// super-sample entries are made once per block (they took a third of the time when
+// each row made its own); eight entries per thread, one node and 16-byte stores
+// where N_M is a multiple of 8.  Bound by the table's reads from L2 and the rows'
+// writes: M = 6375, K' = 12416 (317 MB written) 180 -> 84 us, M = 12944, K' =
+// 33024 (1.7 GB) 753 -> 393 us; trispectrum rows 3240 x 32768 178 -> 101 us.
+struct SplitRows {
+  int64_t rows;
+  int nl, nt, nchi, nm, Kp, nssc, nleg;
+  double sqrt_omega;
+  const int32_t* rd;
+  const double *W, *Mx, *wchi, *sigw2, *chi, *RP3, *RB3;
+  const float* F;
+  const int* E;
+  __nv_bfloat16 *hi, *lo;
+  double* rscale;
+};
+
+template <bool TRI>
+__global__ void __launch_bounds__(256) k_rows_split(SplitRows A) {
+  extern __shared__ double rs_sh[];
+  __shared__ unsigned long long red[8];
+  const int nchi = A.nchi, nm = A.nm, nssc = TRI ? 0 : A.nssc;
+  const int K = nchi * nm, Kt = K + nssc, nk = A.Kp / TW_BK;
+  double* sP = rs_sh;          // [nchi] sqrt(w sigma_W^2) / chi^2, the P rows' super-sample factor
+  double* sB = sP + nchi;      // [nchi] ... / chi^4, the B rows'
+  double* wsh = sB + nchi;     // [nchi] kernel products
+  double* ssh = wsh + nchi;    // [nchi] super-sample entries
+  float* wf = (float*)(ssh + nchi);
+  float* sf = wf + nchi;
+  for (int n = threadIdx.x; n < nssc; n += blockDim.x) {
+    const double ch = A.chi[n], c2_ = ch * ch, q = sqrt(A.wchi[n] * A.sigw2[n]);
+    sP[n] = q / c2_;
+    sB[n] = q / (c2_ * c2_);
   }
-  int L2 = L1 + (int)(r - base);
-  int b1 = L1 / nt, t1 = L1 % nt, b2 = L2 / nt, t2 = L2 % nt;
-  int lo_b = b1 < b2 ? b1 : b2, hi_b = b1 < b2 ? b2 : b1;
-  int sg = lo_b * nl - lo_b * (lo_b - 1) / 2 + (hi_b - lo_b);
-  const int K = nchi * nm;
-  const double* W1 = W + t1 * nchi;
-  const double* W2 = W + t2 * nchi;
-  const int* Es = E + (size_t)sg * nchi;
-  const double* Ms = Mx + (size_t)sg * nchi;
-  double* wsh = ts_sh;
-  double mx = 0.0;
-  for (int n = threadIdx.x; n < nchi; n += blockDim.x) {
-    double w = W1[n] * W2[n] * sqrt_omega;
-    wsh[n] = w;
-    mx = fmax(mx, fabs(w) * Ms[n]);
+  for (int64_t a = blockIdx.x; a < A.rows; a += gridDim.x) {
+    bool isP = true;
+    int sg, t1, t2, t3 = -1, b1 = 0, bt = 0;
+    if (TRI) {
+      // leg pair a: rows of L1 start at L1 (2 nleg + 1 - L1) / 2
+      const float m = 2.0f * (float)A.nleg + 1.0f;
+      int L1 = (int)(0.5f * (m - sqrtf(fmaxf(m * m - 8.0f * (float)a, 0.0f))));
+      L1 = max(0, min(L1, A.nleg - 1));
+      auto start = [&](int L) { return (int64_t)L * (2 * A.nleg + 1 - L) / 2; };
+      while (L1 > 0 && start(L1) > a) --L1;
+      while (start(L1 + 1) <= a) ++L1;
+      const int L2 = L1 + (int)(a - start(L1));  // L1 <= L2, so its bin is not the larger
+      const int x = L1 / A.nt, y = L2 / A.nt;
+      t1 = L1 % A.nt;
+      t2 = L2 % A.nt;
+      sg = x * A.nl - x * (x - 1) / 2 + (y - x);
+    } else {
+      const int32_t* r = A.rd + 8 * a;
+      isP = r[0] == 0;
+      b1 = r[1];
+      bt = r[7];
+      sg = isP ? b1 : A.nl + bt;
+      t1 = r[4];
+      t2 = r[5];
+      if (!isP) t3 = r[6];
+    }
+    const double *W1 = A.W + (int64_t)t1 * nchi, *W2 = A.W + (int64_t)t2 * nchi;
+    const double* W3 = A.W + (int64_t)(t3 < 0 ? t1 : t3) * nchi;
+    const int* Es = A.E + (size_t)sg * nchi;
+    const double* Ms = A.Mx + (size_t)sg * nchi;
+    // per node: kernel products, super-sample entries, row maximum
+    __syncthreads();  // (sP and sB; the last row's weights have been read)
+    unsigned long long mb = 0;
+    auto top = [&](double x) {
+      const unsigned long long w = (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
+      mb = w > mb ? w : mb;
+    };
+    for (int n = threadIdx.x; n < nchi; n += blockDim.x) {
+      double w = W1[n] * W2[n];
+      if (TRI) w *= A.sqrt_omega;
+      if (!TRI && !isP) w *= W3[n];
+      wsh[n] = w;
+      top(w * Ms[n]);
+      if (n < nssc) {
+        const double v = isP ? w * sP[n] * A.RP3[b1 * nchi + n] : w * sB[n] * A.RB3[(int64_t)bt * nchi + n];
+        ssh[n] = v;
+        top(v);
+      }
+    }
+    {
+      const unsigned hi = __reduce_max_sync(~0u, (unsigned)(mb >> 32));
+      const unsigned lo = __reduce_max_sync(~0u, (unsigned)(mb >> 32) == hi ? (unsigned)mb : 0u);
+      if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ((unsigned long long)hi << 32) | lo;
+    }
+    __syncthreads();
+    mb = red[0];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) mb = red[w] > mb ? red[w] : mb;
+    const double mx = __longlong_as_double((long long)mb);
+    int ex = 0;
+    if (mx > 0.0) frexp(mx, &ex);
+    // per node: FP32 weights relative to the row scale 2^ex
+    for (int n = threadIdx.x; n < nchi; n += blockDim.x) {
+      wf[n] = f32_shifted(wsh[n], ex - Es[n]);
+      if (n < nssc) sf[n] = f32_shifted(ssh[n], ex);
+    }
+    if (threadIdx.x == 0) A.rscale[a] = ldexp(1.0, ex);
+    __syncthreads();
+    // per entry: one FP32 product, BF16 hi/lo split
+    const float* Fs = A.F + (size_t)sg * K;
+    for (int kk = 8 * threadIdx.x; kk < A.Kp; kk += 8 * 256) {
+      float x[8];
+      if ((nm & 7) == 0 && kk < K) {
+        const float w = wf[(unsigned)kk / (unsigned)nm];
+        const float4 f0 = __ldg((const float4*)(Fs + kk)), f1 = __ldg((const float4*)(Fs + kk) + 1);
+        x[0] = f0.x * w, x[1] = f0.y * w, x[2] = f0.z * w, x[3] = f0.w * w;
+        x[4] = f1.x * w, x[5] = f1.y * w, x[6] = f1.z * w, x[7] = f1.w * w;
+      } else {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const int k1 = kk + j;
+          x[j] = k1 < K ? Fs[k1] * wf[(unsigned)k1 / (unsigned)nm] : k1 < Kt ? sf[k1 - K] : 0.0f;
+        }
+      }
+      uint32_t h[4], l[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const __nv_bfloat162 h2 = __floats2bfloat162_rn(x[2 * j], x[2 * j + 1]);
+        const __nv_bfloat162 l2 =
+            __floats2bfloat162_rn(x[2 * j] - __low2float(h2), x[2 * j + 1] - __high2float(h2));
+        h[j] = *(const uint32_t*)&h2;
+        l[j] = *(const uint32_t*)&l2;
+      }
+      const int64_t o = blk_off(a, kk, nk);
+      *(uint4*)(A.hi + o) = make_uint4(h[0], h[1], h[2], h[3]);
+      *(uint4*)(A.lo + o) = make_uint4(l[0], l[1], l[2], l[3]);
+    }
   }
-  mx = warp_max(mx);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double t = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
-    t = warp_max(t);
-    if (threadIdx.x == 0) red[0] = t;
-  }
-  __syncthreads();
-  mx = red[0];
-  int ex = 0;
-  if (mx > 0.0) frexp(mx, &ex);
-  float* wf = (float*)(ts_sh + nchi);
-  for (int n = threadIdx.x; n < nchi; n += blockDim.x) wf[n] = (float)ldexp(wsh[n], Es[n] - ex);
-  __syncthreads();
-  const float* Fs = F + (size_t)sg * K;
-  const int nk = Kp / TW_BK;
-  for (int kk = 2 * threadIdx.x; kk < Kp; kk += 2 * blockDim.x) {
-    float x0 = kk < K ? Fs[kk] * wf[(unsigned)kk / (unsigned)nm] : 0.0f;
-    float x1 = kk + 1 < K ? Fs[kk + 1] * wf[(unsigned)(kk + 1) / (unsigned)nm] : 0.0f;
-    __nv_bfloat162 h2 = __floats2bfloat162_rn(x0, x1);
-    __nv_bfloat162 l2 = __floats2bfloat162_rn(x0 - __low2float(h2), x1 - __high2float(h2));
-    int64_t o = blk_off(r, kk, nk);
-    *(__nv_bfloat162*)(hi + o) = h2;
-    *(__nv_bfloat162*)(lo + o) = l2;
-  }
-  if (threadIdx.x == 0) rscale[r] = ldexp(1.0, ex);
 }
 
 // ---------------------------------------------------------------- PTX helpers
@@ -1009,6 +1059,30 @@ static int zero_last_tile(cov_handle* h, void* base, int64_t rows, int K, cudaSt
   return COV_OK;
 }
 
+static int launch_sig(cov_handle* h, int nsig, float* F, int* E, double* Mx, int pairs, cudaStream_t s) {
+  const int per = sig_per_warp(nsig, h->nchi);
+  k_rows_sig<<<dim3((unsigned)((nsig + 8 * per - 1) / (8 * per)), (unsigned)h->nchi), 256, 0, s>>>(
+      h->nl, nsig, h->nchi, h->nm, per, h->tris_d, h->U, h->G2, h->G3, h->C2, h->C3, F, E, Mx, pairs);
+  WL_LAUNCH(h, "k_rows_sig");
+  return COV_OK;
+}
+
+template <bool TRI>
+static int launch_split(cov_handle* h, const SplitRows& A, cudaStream_t s) {
+  const size_t per_node = 4 * sizeof(double) + 2 * sizeof(float);  // 160 KB at N_chi = 4096
+  static std::once_flag attr_once[WL_MAX_DEVICES];
+  static int attr_rc[WL_MAX_DEVICES];
+  if (wl_once_per_device(attr_once, attr_rc, [] {
+        return (int)cudaFuncSetAttribute(k_rows_split<TRI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         4096 * (4 * sizeof(double) + 2 * sizeof(float)));
+      }) != 0)
+    return wl_fail(h, COV_ERR_CUDA, "cudaFuncSetAttribute(k_rows_split) failed");
+  const int64_t grid = std::min<int64_t>(A.rows, 8 * (int64_t)wl_num_sms());
+  if (grid > 0) k_rows_split<TRI><<<(unsigned)grid, 256, A.nchi * per_node, s>>>(A);
+  WL_LAUNCH(h, "k_rows_split");
+  return COV_OK;
+}
+
 int wl_rows_split(cov_handle* h, int nssc, cudaStream_t s) {
   int Kt = h->K + nssc;
   int nsig = h->nl + h->ntri;
@@ -1023,23 +1097,11 @@ int wl_rows_split(cov_handle* h, int nssc, cudaStream_t s) {
   k_rows_prep<<<(h->K + 255) / 256, 256, 0, s>>>(h->nchi, h->nm, 1.0 / h->omega, h->cosmo_d, h->chi, h->wchi,
                                                  h->m, h->om, h->f, h->G2, h->G3, h->C2, h->C3);
   WL_LAUNCH(h, "k_rows_prep");
-  k_rows_sig<<<dim3((unsigned)nsig, (unsigned)h->nchi), 128, 0, s>>>(h->nl, h->ntri, h->nchi, h->nm, h->tris_d, h->U,
-                                                                     h->G2, h->G3, h->C2, h->C3, h->Fsig, h->Esig,
-                                                                     h->Msig, 0);
-  WL_LAUNCH(h, "k_rows_sig");
-  size_t smem = (size_t)h->nchi * (2 * sizeof(double) + 2 * sizeof(float));  // <= 96 KB for N_chi <= 4096
-  static std::once_flag attr_once[WL_MAX_DEVICES];
-  static int attr_rc[WL_MAX_DEVICES];
-  if (wl_once_per_device(attr_once, attr_rc, [] {
-        return (int)cudaFuncSetAttribute(k_rows_split, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         4096 * (2 * sizeof(double) + 2 * sizeof(float)));
-      }) != 0)
-    return wl_fail(h, COV_ERR_CUDA, "cudaFuncSetAttribute(k_rows_split) failed");
-  k_rows_split<<<(unsigned)h->M, 256, smem, s>>>(h->M, h->nl, h->nchi, h->nm, kpad(Kt), nssc, h->rowdesc_d, h->W,
-                                                  h->Fsig, h->Esig, h->Msig, h->wchi, h->sigw2, h->chi, h->RP3,
-                                                  h->RB3, (__nv_bfloat16*)h->Ahi, (__nv_bfloat16*)h->Alo,
-                                                  (double*)h->Ascale);
-  WL_LAUNCH(h, "k_rows_split");
+  if ((rc = launch_sig(h, nsig, h->Fsig, h->Esig, h->Msig, 0, s))) return rc;
+  SplitRows A{h->M,      h->nl,  h->nt,   h->nchi, h->nm,   kpad(Kt), nssc,   h->nleg, 1.0,
+              h->rowdesc_d, h->W, h->Msig, h->wchi, h->sigw2, h->chi,  h->RP3, h->RB3,  h->Fsig, h->Esig,
+              (__nv_bfloat16*)h->Ahi, (__nv_bfloat16*)h->Alo, (double*)h->Ascale};
+  if ((rc = launch_split<false>(h, A, s))) return rc;
   return COV_OK;
 }
 
@@ -1063,15 +1125,11 @@ int wl_trows_split(cov_handle* h, cudaStream_t s) {
   k_rows_prep<<<(h->K + 255) / 256, 256, 0, s>>>(h->nchi, h->nm, 1.0 / h->omega, h->cosmo_d, h->chi, h->wchi,
                                                  h->m, h->om, h->f, h->G2, h->G3, h->C2, h->C3);
   WL_LAUNCH(h, "k_rows_prep");
-  k_rows_sig<<<dim3((unsigned)npair, (unsigned)h->nchi), 128, 0, s>>>(h->nl, h->ntri, h->nchi, h->nm, h->tris_d, h->U,
-                                                                      h->G2, h->G3, h->C2, h->C3, h->FsigT, h->EsigT,
-                                                                      h->MsigT, 1);
-  WL_LAUNCH(h, "k_rows_sig");
-  size_t smem = (size_t)h->nchi * (sizeof(double) + sizeof(float));
-  k_trows_split<<<(unsigned)h->ntrow, 256, smem, s>>>(h->ntrow, h->nleg, h->nt, h->nl, h->nchi, h->nm, kpad(h->K),
-                                                       sqrt(h->omega), h->W, h->FsigT, h->EsigT, h->MsigT,
-                                                       (__nv_bfloat16*)h->Thi, (__nv_bfloat16*)h->Tlo, h->Tscale);
-  WL_LAUNCH(h, "k_trows_split");
+  if ((rc = launch_sig(h, npair, h->FsigT, h->EsigT, h->MsigT, 1, s))) return rc;
+  SplitRows A{h->ntrow,  h->nl,  h->nt,    h->nchi, h->nm,   kpad(h->K), 0,      h->nleg, sqrt(h->omega),
+              h->rowdesc_d, h->W, h->MsigT, h->wchi, h->sigw2, h->chi,    h->RP3, h->RB3,  h->FsigT, h->EsigT,
+              (__nv_bfloat16*)h->Thi, (__nv_bfloat16*)h->Tlo, h->Tscale};
+  if ((rc = launch_split<true>(h, A, s))) return rc;
   return COV_OK;
 }
 
