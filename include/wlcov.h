@@ -371,7 +371,9 @@ int cov_pca(cov_handle* h, const double* d_C, int64_t ldc, const double* d_D, do
  * graph, the step is captured alone and replayed once per cosmology
  * (info->single_launch tells which).  The exact counts are computed once.  Results equal those of cov_update + cov_spectra +
  * cov_assemble + cov_snr for each cosmology.  The handle keeps a dense M x M
- * covariance and the (M + 1)^2 Cholesky workspace.  A non-positive pivot or an
+ * covariance and the (M + 1)^2 Cholesky workspace; without a memory budget the
+ * P and B factorisations of mid-sized row sets run beside the joint one, in a
+ * second workspace that is given back on return.  A non-positive pivot or an
  * expired wait in any cosmology fails the whole batch (COV_ERR_NOT_PD /
  * COV_ERR_TIMEOUT).  Afterwards the handle holds the last cosmology. */
 #define COV_BATCH_TUNE 1u

@@ -14,21 +14,13 @@
 // graph launch (fallback: the step captured alone and replayed per
 // cosmology).  The exact integer counts do not depend on the cosmology and are
 // computed once.
+#include <algorithm>
 #include <chrono>
+#include <utility>
 
 #include "common.cuh"
 
 namespace {
-
-// one eager step for the handle's current cosmology (tables already built)
-int eager_step(cov_handle* h, unsigned terms, int precision, double* C, double* D, double* snr3, cudaStream_t s) {
-  int rc;
-  if ((rc = wl_spectra(h, D, s))) return rc;
-  if ((rc = wl_assemble(h, C, h->M, terms, precision, s))) return rc;
-  for (int w = 0; w < 3; ++w)
-    if ((rc = wl_snr(h, C, h->M, D, w, snr3 + (size_t)w * h->nl, s))) return rc;
-  return COV_OK;
-}
 
 struct Pinned {
   void* p = nullptr;
@@ -43,6 +35,110 @@ struct DevBuf {
     if (p) cudaFree(p);
   }
 };
+
+// A second set of what a factorisation works in: the P and B factorisations of a
+// step run beside the joint one.  Each is a chain of panels that leaves most of
+// the device idle: the three of M = 3064 take
+// 5.6 ms in turn and 3.1 ms so.  For the
+// call only: it is given back when the call returns.
+#define LANE_MIN_ROWS 2048  // rows of all cosmologies: ~0.7 us saved for each, ~0.4 ms to set up
+#define LANE_MAX_ROWS 8192  // beyond, the updates fill the device (and the copy is > 0.5 GB)
+struct Lane {
+  DevBuf work, scratch;
+  int64_t work_n = 0;
+  size_t scratch_n = 0;
+  cudaStream_t s = nullptr, side = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr, cols = nullptr, panel = nullptr;
+  bool ok = false;
+  ~Lane() {
+    for (cudaEvent_t e : {fork, join, cols, panel})
+      if (e) cudaEventDestroy(e);
+    for (cudaStream_t t : {s, side})
+      if (t) cudaStreamDestroy(t);
+  }
+};
+
+// Not with a memory budget, for large matrices, or
+// when anything fails: the factorisations then run in turn.
+void make_lane(cov_handle* h, int n, Lane* l) {
+  const int64_t Ms = std::max(h->sel[COV_WHICH_P].Ms, h->sel[COV_WHICH_B].Ms);
+  if (h->budget || h->chol_scratch_cap || Ms * n < LANE_MIN_ROWS || Ms > LANE_MAX_ROWS) return;
+  l->work_n = (Ms + 1 + 7) / 8 * 8 * (Ms + 1);
+  l->scratch_n = wl_fx_bytes(Ms, 4);
+  size_t free_b = 0, total_b = 0;
+  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || free_b < 4 * (sizeof(double) * l->work_n + l->scratch_n)) {
+    cudaGetLastError();
+    return;
+  }
+  int least = 0, greatest = 0;
+  auto good = [](cudaError_t e) { return e == cudaSuccess; };
+  l->ok = good(cudaMalloc(&l->work.p, sizeof(double) * l->work_n)) && good(cudaMalloc(&l->scratch.p, l->scratch_n)) &&
+          good(cudaDeviceGetStreamPriorityRange(&least, &greatest)) &&
+          good(cudaStreamCreateWithPriority(&l->s, cudaStreamNonBlocking, least)) &&
+          good(cudaStreamCreateWithPriority(&l->side, cudaStreamNonBlocking, greatest));
+  for (cudaEvent_t* e : {&l->fork, &l->join, &l->cols, &l->panel})
+    l->ok = l->ok && good(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+  if (!l->ok) cudaGetLastError();
+}
+
+// the three factorisations of a step, enqueued (h->deferred)
+int snr_three(cov_handle* h, Lane* l, cudaStream_t s) {
+  const int64_t M = h->M;
+  int rc = COV_OK;
+  if (!l->ok) {
+    for (int w = 0; w < 3 && !rc; ++w) rc = wl_snr(h, h->batch_C, M, h->batch_D, w, nullptr, s);
+    return rc;
+  }
+  WL_CHECK(h, cudaEventRecord(l->fork, s));
+  WL_CHECK(h, cudaStreamWaitEvent(l->s, l->fork, 0));
+  auto swap_in = [&] {
+    double* const w = h->work;
+    h->work = (double*)l->work.p;
+    l->work.p = w;
+    std::swap(h->work_n, l->work_n);
+    std::swap(h->chol_scratch, l->scratch.p);
+    std::swap(h->chol_scratch_n, l->scratch_n);
+    std::swap(h->side, l->side);
+    std::swap(h->ev_cols, l->cols);
+    std::swap(h->ev_panel, l->panel);
+  };
+  const int64_t ld = h->work_ld;
+  swap_in();
+  for (int w : {COV_WHICH_P, COV_WHICH_B})
+    if (!rc) rc = wl_snr(h, h->batch_C, M, h->batch_D, w, nullptr, l->s);
+  swap_in();  // back
+  h->work_ld = ld;
+  if (!rc) rc = wl_snr(h, h->batch_C, M, h->batch_D, COV_WHICH_JOINT, nullptr, s);
+  WL_CHECK(h, cudaEventRecord(l->join, l->s));
+  WL_CHECK(h, cudaStreamWaitEvent(s, l->join, 0));
+  return rc;
+}
+
+// one eager step for the handle's current cosmology (tables already built)
+int eager_step(cov_handle* h, unsigned terms, int precision, double* C, double* D, double* snr3, Lane* lane,
+               cudaStream_t s) {
+  int rc;
+  if ((rc = wl_spectra(h, D, s))) return rc;
+  if ((rc = wl_assemble(h, C, h->M, terms, precision, s))) return rc;
+  if (!lane->ok) {
+    for (int w = 0; w < 3; ++w)
+      if ((rc = wl_snr(h, C, h->M, D, w, snr3 + (size_t)w * h->nl, s))) return rc;
+    return COV_OK;
+  }
+  for (int* w : {h->chol_status, h->piv_status}) WL_CHECK(h, cudaMemsetAsync(w, 0, sizeof(int), s));
+  h->deferred = true;
+  rc = snr_three(h, lane, s);
+  h->deferred = false;
+  if (rc) return rc;
+  for (int w = 0; w < 3; ++w) {
+    if (h->sel[w].Ms)
+      WL_CHECK(h, cudaMemcpyAsync(snr3 + (size_t)w * h->nl, h->sel[w].out, sizeof(double) * h->nl,
+                                  cudaMemcpyDeviceToHost, s));
+    else
+      std::fill(snr3 + (size_t)w * h->nl, snr3 + (size_t)(w + 1) * h->nl, nan(""));
+  }
+  return wl_snr_status(h, s);
+}
 
 // Loop body, first kernel: the cosmology of iteration *idx into the copy the
 // kernels of the step read.
@@ -78,7 +174,8 @@ __global__ void k_batch_out(int* idx, int n, int nl, int64_t M, const double* s0
 // body is k_batch_in, the captured step and k_batch_out.  *built is false when
 // the graph could not be built (the caller then replays the step per cosmology).
 int single_launch(cov_handle* h, const cov_cosmology* cosmos, int n, unsigned terms, int precision, bool with_D,
-                  double* out_host, size_t per, cudaStream_t s, double* cap_ms, double* run_ms, bool* built) {
+                  double* out_host, size_t per, Lane* lane, cudaStream_t s, double* cap_ms, double* run_ms,
+                  bool* built) {
   *built = false;
   const int64_t M = h->M;
   DevBuf dc, dout, didx;
@@ -124,7 +221,7 @@ int single_launch(cov_handle* h, const cov_cosmology* cosmos, int n, unsigned te
       rc = wl_tables(h, s);
       if (!rc) rc = wl_spectra(h, h->batch_D, s);
       if (!rc) rc = wl_assemble(h, h->batch_C, M, terms, precision, s);
-      for (int w = 0; w < 3 && !rc; ++w) rc = wl_snr(h, h->batch_C, M, h->batch_D, w, nullptr, s);
+      if (!rc) rc = snr_three(h, lane, s);
       k_batch_out<<<1, 256, 0, s>>>((int*)didx.p, n, h->nl, M, h->sel[0].out, h->sel[1].out, h->sel[2].out,
                                     with_D ? h->batch_D : nullptr, (double*)dout.p, (int64_t)per, loop);
       cudaGraph_t captured = nullptr;
@@ -182,6 +279,9 @@ extern "C" int cov_batch_snr(cov_handle* h, const cov_cosmology* cosmos, int n, 
     return std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t).count();
   };
 
+  if ((rc = wl_snr_prepare(h, s))) return rc;
+  Lane lane;
+  make_lane(h, n, &lane);
   // 1. the first cosmology, eagerly (optionally once per candidate configuration)
   auto t0 = std::chrono::steady_clock::now();
   if ((rc = cov_update(h, &cosmos[0], s))) return rc;
@@ -205,7 +305,7 @@ extern "C" int cov_batch_snr(cov_handle* h, const cov_cosmology* cosmos, int n, 
       h->chol_kernel = cands[a].chol;
       WL_CHECK(h, cudaStreamSynchronize(s));
       auto t = std::chrono::steady_clock::now();
-      if ((rc = eager_step(h, terms, precision, h->batch_C, h->batch_D, h_snr, s))) return rc;
+      if ((rc = eager_step(h, terms, precision, h->batch_C, h->batch_D, h_snr, &lane, s))) return rc;
       WL_CHECK(h, cudaStreamSynchronize(s));
       const double ms = ms_since(t);
       inf.candidate_ms[a] = ms;
@@ -220,7 +320,7 @@ extern "C" int cov_batch_snr(cov_handle* h, const cov_cosmology* cosmos, int n, 
     h->chol_kernel = cands[bi].chol;
     inf.tuned = bi;
   }
-  if ((rc = eager_step(h, terms, precision, h->batch_C, h->batch_D, h_snr, s))) return rc;
+  if ((rc = eager_step(h, terms, precision, h->batch_C, h->batch_D, h_snr, &lane, s))) return rc;
   if (h_D) WL_CHECK(h, cudaMemcpyAsync(h_D, h->batch_D, sizeof(double) * M, cudaMemcpyDeviceToHost, s));
   WL_CHECK(h, cudaStreamSynchronize(s));
   inf.first_ms = ms_since(t0);
@@ -241,7 +341,8 @@ extern "C" int cov_batch_snr(cov_handle* h, const cov_cosmology* cosmos, int n, 
     // 2. cosmologies 1..n-1 as one graph launch (a device-side loop)
     bool built = false;
     double cap_ms = 0.0, run_ms = 0.0;
-    if ((rc = single_launch(h, cosmos, n, terms, precision, h_D != nullptr, out, per, s, &cap_ms, &run_ms, &built)))
+    if ((rc = single_launch(h, cosmos, n, terms, precision, h_D != nullptr, out, per, &lane, s, &cap_ms, &run_ms,
+                            &built)))
       return rc;
     if (built) {
       inf.single_launch = 1;
@@ -258,7 +359,7 @@ extern "C" int cov_batch_snr(cov_handle* h, const cov_cosmology* cosmos, int n, 
       rc = wl_tables(h, s);
       if (!rc) rc = wl_spectra(h, h->batch_D, s);
       if (!rc) rc = wl_assemble(h, h->batch_C, M, terms, precision, s);
-      for (int w = 0; w < 3 && !rc; ++w) rc = wl_snr(h, h->batch_C, M, h->batch_D, w, nullptr, s);
+      if (!rc) rc = snr_three(h, &lane, s);
       ce = cudaStreamEndCapture(s, &graph);
       h->deferred = false;
       h->prof = prof;

@@ -147,8 +147,13 @@ static int factor_and_prefix(cov_handle* h, OutMap Wm, int64_t Ms, const int* pe
   WL_LAUNCH(h, "k_snr_prefix");
   wl_stage_end(h, tk, s);
   if (h->deferred) return COV_OK;
-  int status = 0, tstatus = 0;
   WL_CHECK(h, cudaMemcpyAsync(h_snr, out_d, sizeof(double) * h->nl, cudaMemcpyDeviceToHost, s));
+  return wl_snr_status(h, s);
+}
+
+// The status words of the factorisations on s (synchronises it)
+int wl_snr_status(cov_handle* h, cudaStream_t s) {
+  int status = 0, tstatus = 0;
   WL_CHECK(h, cudaMemcpyAsync(&status, h->piv_status, sizeof(int), cudaMemcpyDeviceToHost, s));
   WL_CHECK(h, cudaMemcpyAsync(&tstatus, h->chol_status, sizeof(int), cudaMemcpyDeviceToHost, s));
   WL_CHECK(h, cudaStreamSynchronize(s));
@@ -196,6 +201,15 @@ static int selection(cov_handle* h, int slot, cudaStream_t s) {
   WL_CHECK(h, cudaStreamSynchronize(s));  // sel and cnt are host memory read by the copies
   z.Ms = Ms;
   z.ready = true;
+  return COV_OK;
+}
+
+// What a step with deferred status reads needs first: the selections and status words
+int wl_snr_prepare(cov_handle* h, cudaStream_t s) {
+  int rc;
+  for (int w = 0; w < 3; ++w)
+    if ((rc = selection(h, w, s))) return rc;
+  if (!h->chol_status) WL_CHECK(h, cudaMalloc(&h->chol_status, sizeof(int)));
   return COV_OK;
 }
 

@@ -290,6 +290,8 @@ int wl_assemble(cov_handle* h, double* d_C, int64_t ldc, unsigned terms, int pre
 int wl_snr_tiles(cov_handle* h, double* Ct, const double* D, double* h_snr, cudaStream_t s);  // chol.cu
 int wl_assemble_band(cov_handle* h, int64_t row0, int64_t nrows, OutMap out, unsigned terms, int precision,
                      cudaStream_t s);
+int wl_snr_prepare(cov_handle* h, cudaStream_t s);  // chol.cu
+int wl_snr_status(cov_handle* h, cudaStream_t s);   // chol.cu
 int wl_snr(cov_handle* h, const double* d_C, int64_t ldc, const double* d_D, int which, double* h_snr,
            cudaStream_t s, const int* perm = nullptr);  // chol.cu
 int wl_gemm_lower_fp64(cov_handle* h, const double* A, int64_t lda, const double* B, int64_t ldb, double* C,
