@@ -329,6 +329,22 @@ size_t wl_chol_scratch_est(int64_t n) {
   return (pad * 772 + 255) / 256 * 256;
 }
 
+// Upper bound of what a handle may still allocate on demand in its other calls (both
+// forms' operands, the batch's covariance, the Cholesky and PCA workspaces): a larger,
+// faster form of a buffer is taken only where all of this fits beside it, so that no
+// call is refused for it.
+size_t wl_late_bytes(const cov_handle* h) {
+  const size_t M = (size_t)h->M, K = (size_t)h->K, nchi = (size_t)h->nchi, nt = (size_t)h->ntrow, nl = (size_t)h->nl;
+  const size_t Mp = (M + 255) / 256 * 256, tp = (nt + 255) / 256 * 256, Kp = K + nchi + 64;
+  const size_t t = (std::max(M, nt) + 255) / 256 + 1, nb32 = (M + 31) / 32;
+  size_t b = 3 * M * M * 8 + 32 * M * 8;                                    // covariance, Cholesky, PCA
+  b += M * Kp * 8 + nt * K * 8 + nt * nt * 8;                               // FP64 rows, trispectrum table
+  b += 4 * (Mp + tp) * Kp + (nl + (size_t)h->ntri + nl * (nl + 1) / 2) * (K * 4 + nchi * 12);  // split rows, signatures
+  b += 2 * wl_chol_scratch_est((int64_t)M + 1) + WL_TILE_CACHE * (t * (t + 1) / 2) * 8 + nb32 * (nb32 + 1) / 2 * 4;
+  if (h->coupling == COV_COUPLING_EXACT) b *= 2;  // (and the exact couplings' transients)
+  return b + 2 * wl_coupling_bytes(h) + ((size_t)64 << 20);
+}
+
 // Host-only upper estimate of the device bytes one request holds at its peak:
 // the handle's tables, the dense covariance and data vector, the contraction
 // operands of the chosen precision, the trispectrum table, the Cholesky

@@ -27,8 +27,8 @@
 // What bounds it: up to M ~ 10000 the chain of panels (M = 6375: 100 panels of ~45 us
 // and their ~12 us inner updates of the 7.7 ms), beyond that the passes over the entries
 // and the exact sums' additions in the updates' epilogue (M = 24400: 156 ms).  Against
-// FP64 diagonal blocks and panel solves: the three S/N of M = 6375 14.4 -> 7.9 ms, of
-// M = 818 1.28 -> 0.80 ms, the one in place at M = 24400 268 -> 158 ms.
+// FP64 diagonal blocks and panel solves: the joint S/N of M = 6375 14.4 -> 7.9 ms, of
+// M = 818 1.28 -> 0.78 ms, the one in place at M = 24400 268 -> 158 ms.
 //
 // Error: entries 2^-63 by rounding, updates 2^-56 per digit row against the unit
 // diagonal, i.e. below that of an FP64 factorisation (2^-53 per operation).
@@ -69,6 +69,23 @@ __device__ __forceinline__ long long fx_fixed(double x, int* status) {
     q += (rem > half || (rem == half && (q & 1ull))) ? 1ull : 0ull;
   }
   return (b >> 63) ? -(long long)q : (long long)q;
+}
+
+// two neighbouring entries; `wide`: the pair is 16-byte aligned (COV_CHOL_TILE also takes
+// packed tiles that are not)
+__device__ __forceinline__ ulonglong2 fx_ld2(const double* p, int wide) {
+  if (wide) return *(const ulonglong2*)p;
+  const unsigned long long* q = (const unsigned long long*)p;
+  return make_ulonglong2(q[0], q[1]);
+}
+__device__ __forceinline__ void fx_st2(double* p, unsigned long long a, unsigned long long b, int wide) {
+  if (wide) {
+    *(ulonglong2*)p = make_ulonglong2(a, b);
+  } else {
+    unsigned long long* q = (unsigned long long*)p;
+    q[0] = a;
+    q[1] = b;
+  }
 }
 
 // ---------------------------------------------------------------- scaling
@@ -229,6 +246,7 @@ struct FxPanel {
   uint8_t* dig;
   double *y, *ld, *ld_prev;  // solved data vector; this and the previous panel's diagonal factor (64 x 64)
   int* status;
+  int wide;  // the matrix is 16-byte aligned
 };
 
 // 1 / L_jj from the pivot's r (as two halves) and shift
@@ -436,7 +454,9 @@ __global__ void __maxnreg__(104) k_fx_panel(FxPanel P) {
     for (int t = 0; t < SL_S; ++t) *(uint4*)(o + (size_t)t * SL_DIGIT) = d[t];
     double* rowp = W.at(row, k0) + 8 * q;  // 64 consecutive entries (k0 is a multiple of 64)
 #pragma unroll
-    for (int p = 0; p < 8; p += 2) *(double2*)(rowp + p) = make_double2(xd[p], xd[p + 1]);
+    for (int p = 0; p < 8; p += 2)
+      fx_st2(rowp + p, (unsigned long long)__double_as_longlong(xd[p]),
+             (unsigned long long)__double_as_longlong(xd[p + 1]), P.wide);
     if (q == 0) *W.at(P.Ms, row) -= dot;
   }
 }
@@ -485,6 +505,7 @@ struct FxUpd {
   FxTiles t;
   int64_t ntiles;
   int* status;
+  int wide;  // the matrix is 16-byte aligned
 };
 
 // A CTA takes every gridDim-th tile of 128 x 64.  The accumulators start as the tile's
@@ -546,7 +567,7 @@ __global__ void __maxnreg__(120)
         for (int c = 0; c < 16; c += 2) {
           const int u = ((c >> 1) & 1) + 2 * (c >> 3), o = j * SL_BN + 8 * ((c >> 2) & 1);
           ulonglong2 v = make_ulonglong2(0ull, 0ull);
-          if (o <= nc[u]) v = *(const ulonglong2*)(p[u] + o);
+          if (o <= nc[u]) v = fx_ld2(p[u] + o, A.wide);
           acc[j][c] = v.x - off;
           acc[j][c + 1] = v.y - off;
         }
@@ -556,7 +577,7 @@ __global__ void __maxnreg__(120)
 #pragma unroll
         for (int c = 0; c < 16; c += 2) {
           const int u = ((c >> 1) & 1) + 2 * (c >> 3), o = j * SL_BN + 8 * ((c >> 2) & 1);
-          if (o <= nc[u]) *(ulonglong2*)(p[u] + o) = make_ulonglong2(acc[j][c], acc[j][c + 1]);
+          if (o <= nc[u]) fx_st2(p[u] + o, acc[j][c], acc[j][c + 1], A.wide);
         }
     }
   }
@@ -600,6 +621,14 @@ static int fx_scratch(cov_handle* h, int64_t n, int* w_out) {
       *w_out = w;
       return COV_OK;
     }
+    if (w > 1) {
+      if (h->deferred && h->chol_scratch) continue;  // (a captured step keeps to what the eager one allocated)
+      size_t fr = 0, tot = 0;
+      const bool known = cudaMemGetInfo(&fr, &tot) == cudaSuccess;
+      if (!known || need > fr / 16 ||
+          (h->budget && h->allocated - h->chol_scratch_n + need + wl_late_bytes(h) > h->budget))
+        continue;
+    }
     void* p = nullptr;
     cudaError_t e = cudaMalloc(&p, need);
     if (e != cudaSuccess) {
@@ -642,11 +671,13 @@ static int fx_attributes(cov_handle* h) {
   return COV_OK;
 }
 
+static int fx_wide(const OutMap& W) { return ((uintptr_t)W.C & 15) == 0 && (W.tiled || W.ldc % 2 == 0); }
+
 // columns [c0, c1) of the trailing matrix of rows c0 .. Ms - 1, on at most `sms` SMs
 static int fx_update(cov_handle* h, OutMap W, int64_t Ms, int64_t rb0, int kblk, int nk, int nkb, int64_t c0, int64_t c1,
                      const FxMaps& m, int64_t sms, cudaStream_t s) {
   if (c0 >= c1 || c0 >= Ms) return COV_OK;
-  FxUpd a{W, Ms, rb0, kblk, nk, nkb, {}, 0, h->chol_status};
+  FxUpd a{W, Ms, rb0, kblk, nk, nkb, {}, 0, h->chol_status, fx_wide(W)};
   a.t.j0 = c0 / 64;
   a.t.nj = (c1 + 63) / 64 - a.t.j0;
   a.t.i0 = c0 / SL_BM;
@@ -666,7 +697,7 @@ static int fx_update(cov_handle* h, OutMap W, int64_t Ms, int64_t rb0, int kblk,
 int wl_fx_factor(cov_handle* h, OutMap W, int64_t Ms, const int* perm, const double* C, int64_t ldc, const double* D,
                  cudaStream_t s) {
   int rc, w = 4;
-  if (((uintptr_t)W.C & 15) != 0 || (!W.tiled && W.ldc % 2 != 0))
+  if (h->chol_kernel != 1 && !fx_wide(W))
     return wl_fail(h, COV_ERR_CUDA, "Cholesky: the matrix is not 16-byte aligned");
   if ((rc = fx_attributes(h))) return rc;
   if ((rc = fx_scratch(h, Ms, &w))) return rc;
@@ -703,7 +734,7 @@ int wl_fx_factor(cov_handle* h, OutMap W, int64_t Ms, const int* perm, const dou
       const int64_t k0 = S0 + (int64_t)p * FX_NB;
       const int slot = (int)((k0 / FX_NB) & 1);
       FxPanel a{W, k0, Ms, S0 / SL_BM, (int)std::min<int64_t>(FX_NB, Ms - k0), 2 * p, nkb, fx_dig(h, Ms, w, b), y,
-                ld + slot * FX_NB * FX_NB, ld + (slot ^ 1) * FX_NB * FX_NB, st};
+                ld + slot * FX_NB * FX_NB, ld + (slot ^ 1) * FX_NB * FX_NB, st, fx_wide(W)};
       const int64_t groups = std::max<int64_t>(0, (Ms - k0 - FX_NB + FX_RB - 1) / FX_RB);
       k_fx_panel<<<(unsigned)(groups + 1), FX_THREADS, FX_PSMEM, st_>>>(a);
       WL_LAUNCH(h, "k_fx_panel");

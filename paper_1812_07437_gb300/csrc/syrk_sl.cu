@@ -418,8 +418,9 @@ int wl_sl_rows(cov_handle* h, bool tri, int nssc, cudaStream_t s) {
 
 // Whether the tensor-core FP64 form serves the handle's rows (tri: its trispectrum
 // rows), and its buffers.  The digits take 14 bytes per entry where the FP64 rows of
-// k_gemm_lower take 8; where they do not fit (hbm_budget, or three quarters of the
-// free memory) the FP64 rows and that kernel serve the handle as before.  Decided
+// k_gemm_lower take 8; where they do not fit (in hbm_budget, or the free memory, beside
+// all that the handle's other calls may still allocate) the FP64 rows and that kernel
+// serve the handle as before.  Decided
 // once per handle: a later call with more super-sample columns finds room for them.
 int wl_sl_alloc(cov_handle* h, bool tri, bool* use, cudaStream_t s) {
   int& state = tri ? h->sl_tri : h->sl_rows;
@@ -450,7 +451,8 @@ int wl_sl_alloc(cov_handle* h, bool tri, bool* use, cudaStream_t s) {
     if (!*a.p) need += a.n;
   size_t fr = 0, tot = 0;
   WL_CHECK(h, cudaMemGetInfo(&fr, &tot));
-  bool ok = need <= fr / 4 * 3 && !(h->budget && h->allocated + need > h->budget);
+  const size_t late = wl_late_bytes(h);
+  bool ok = need <= fr / 4 * 3 && need + late <= fr && !(h->budget && h->allocated + need + late > h->budget);
   const bool had_trd = h->trd != nullptr;
   std::vector<void**> got;
   for (auto& a : al) {

@@ -109,3 +109,26 @@ def test_not_positive_definite(nt, nl):
     bad(lambda B: B.__setitem__((M - 1, 0), float(2.0 * d[M - 1] * d[0])))
     assert np.array_equal(h.snr(C, D, N.COV_WHICH_P), good)
     h.close()
+
+
+def test_packed_tiles_off_16_bytes():
+    """COV_CHOL_TILE takes tiles that are only 8-byte aligned, with the same numbers; COV_CHOL_AUTO refuses them."""
+    from paper_1812_07437_gb300.handle import Handle, packed_tiles
+    wl = workloads.get("tiny_2bin")
+    wl["nz"].update(n_tomo=3, photoz_sigma0=0.05)
+    wl["bins"].update(n_ell=6, ell_min=30.0, ell_max=2000.0)
+    out = []
+    for off, kernel in ((0, N.COV_CHOL_TILE), (1, N.COV_CHOL_TILE), (1, N.COV_CHOL_AUTO)):
+        h = Handle(wl, order=N.COV_ORDER_CUMULATIVE, chol_kernel=kernel)
+        D = torch.zeros(h.M, dtype=torch.float64, device=DEV)
+        h.spectra(D)
+        Ct = torch.zeros(packed_tiles(h.M + 1) * 65536 + 1, dtype=torch.float64, device=DEV)[off:]
+        h.assemble_band(0, h.M, Ct, N.COV_LAYOUT_TILES, N.COV_TERMS_ALL, N.COV_FP64)
+        if kernel == N.COV_CHOL_TILE:
+            out.append(h.snr_tiles(Ct, D))
+        else:
+            with pytest.raises(N.CovError) as e:
+                h.snr_tiles(Ct, D)
+            assert e.value.code == N.COV_ERR_CUDA
+        h.close()
+    assert np.array_equal(out[0], out[1], equal_nan=True)
