@@ -311,7 +311,7 @@ static int gemm_lower_band(cov_handle* h, const double* A, int64_t lda, int64_t 
 
 int wl_ensure(cov_handle* h, void** p, size_t bytes, const char* what) {
   if (*p) return COV_OK;
-  if (h->budget && h->allocated + bytes > h->budget)
+  if (wl_over_budget(h, bytes))
     return wl_fail(h, COV_ERR_NOMEM, std::string("hbm_budget exceeded allocating ") + what);
   cudaError_t e = cudaMalloc(p, bytes);
   if (e != cudaSuccess) {

@@ -236,7 +236,7 @@ int wl_snr(cov_handle* h, const double* C, int64_t ldc, const double* D, int whi
     }
     h->work = nullptr;
     h->work_n = 0;
-    if (h->budget && h->allocated + sizeof(double) * need > h->budget)
+    if (wl_over_budget(h, sizeof(double) * need))
       return wl_fail(h, COV_ERR_NOMEM, "hbm_budget exceeded allocating the Cholesky workspace");
     WL_CHECK(h, cudaMalloc(&h->work, sizeof(double) * need));
     h->work_n = need;

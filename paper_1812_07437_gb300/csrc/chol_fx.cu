@@ -626,7 +626,7 @@ static int fx_scratch(cov_handle* h, int64_t n, int* w_out) {
       size_t fr = 0, tot = 0;
       const bool known = cudaMemGetInfo(&fr, &tot) == cudaSuccess;
       if (!known || need > fr / 16 ||
-          (h->budget && h->allocated - h->chol_scratch_n + need + wl_late_bytes(h) > h->budget))
+          (h->budget && h->allocated - h->chol_scratch_n + need + ((size_t)64 << 20) > h->budget))
         continue;
     }
     void* p = nullptr;
@@ -647,6 +647,20 @@ static int fx_scratch(cov_handle* h, int64_t n, int* w_out) {
     return COV_OK;
   }
   return COV_OK;
+}
+
+// Whether `extra` bytes more are beyond the handle's budget.  The Cholesky's scratch is
+// given back first where it stands in the way: it is wider than it has to be, and the
+// next factorisation takes what then fits.
+bool wl_over_budget(cov_handle* h, size_t extra) {
+  if (!h->budget || h->allocated + extra <= h->budget) return false;
+  if (h->chol_scratch && !h->deferred) {
+    cudaFree(h->chol_scratch);
+    h->allocated -= h->chol_scratch_n;
+    h->chol_scratch = nullptr;
+    h->chol_scratch_n = 0;
+  }
+  return h->allocated + extra > h->budget;
 }
 
 static uint8_t* fx_dig(cov_handle* h, int64_t n, int w, int b) {

@@ -315,6 +315,7 @@ size_t wl_handle_bytes(const cov_handle* h);
 void wl_set_global_error(const std::string& msg);  // api.cu: read by cov_last_error(NULL)
 size_t wl_chol_scratch_est(int64_t n);  // api.cu
 size_t wl_late_bytes(const cov_handle* h);  // api.cu: bound of later allocations
+bool wl_over_budget(cov_handle* h, size_t extra);  // chol_fx.cu
 size_t wl_fx_bytes(int64_t n, int w);  // chol_fx.cu: scratch with super-panels of w panels
 int wl_fx_factor(cov_handle* h, OutMap W, int64_t Ms, const int* perm, const double* C, int64_t ldc, const double* D,
                  cudaStream_t s);  // chol_fx.cu

@@ -269,7 +269,7 @@ int wl_couplings(cov_handle* h, cudaStream_t s) {
   const size_t resident = wl_coupling_bytes(h);
   const size_t transient = nm_bytes + sizeof(int2) * orb.size() + sizeof(ColDesc) * cd.size() +
                            (8 + 4) * (size_t)ncol_all + 8 * (size_t)sq;
-  if (h->budget && h->allocated + resident + transient > h->budget)
+  if (wl_over_budget(h, resident + transient))
     return wl_fail(h, COV_ERR_NOMEM, "hbm_budget exceeded by the exact couplings");
   DevTmp d_orb, d_cd, d_nm, d_sum, d_ctri, d_gf, d_bad;
   WL_CHECK(h, cudaMalloc(&d_orb.p, sizeof(int2) * std::max<size_t>(orb.size(), 1)));

@@ -401,7 +401,7 @@ extern "C" int cov_pca(cov_handle* h, const double* d_C, int64_t ldc, const doub
       h->pca_buf = nullptr;
       h->pca_bytes = 0;
     }
-    if (h->budget && h->allocated + need > h->budget)
+    if (wl_over_budget(h, need))
       return wl_fail(h, COV_ERR_NOMEM, "hbm_budget exceeded allocating the PCA workspace");
     WL_CHECK(h, cudaMalloc(&h->pca_buf, need));
     h->pca_bytes = need;

@@ -132,3 +132,29 @@ def test_packed_tiles_off_16_bytes():
             assert e.value.code == N.COV_ERR_CUDA
         h.close()
     assert np.array_equal(out[0], out[1], equal_nan=True)
+
+
+def test_scratch_under_a_budget():
+    """A budget that holds either the wide scratch or a later workspace: the scratch goes, the call is served."""
+    from paper_1812_07437_gb300.handle import Handle
+    wl = workloads.get("mid_3bin")
+    free = Handle(wl)
+    M = free.M
+    C, _, D = _problem(M, False, 11)
+    ref = free.snr(C, D, N.COV_WHICH_JOINT)
+    lam = free.pca(C, D)["lam"]
+    free.close()
+    # what cov_init takes is found as the least accepted budget, in steps of 1 MB
+    for mb in range(1, 4096):
+        try:
+            h = Handle(wl, hbm_budget=mb << 20)
+            break
+        except N.CovError as e:
+            assert e.code == N.COV_ERR_NOMEM
+    h.close()
+    work, pca = (M + 8) * (M + 1) * 8, M * (M + 9) * 8 + 8 * M + 64
+    h = Handle(wl, hbm_budget=(mb << 20) + work + pca + (1 << 20))
+    assert np.array_equal(h.snr(C, D, N.COV_WHICH_JOINT), ref, equal_nan=True)
+    np.testing.assert_array_equal(h.pca(C, D)["lam"], lam)
+    assert np.array_equal(h.snr(C, D, N.COV_WHICH_JOINT), ref, equal_nan=True)
+    h.close()
