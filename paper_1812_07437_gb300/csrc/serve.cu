@@ -42,6 +42,7 @@ struct Rec {
   std::string key, err;
   int bypassed = 0;
   bool digits = false;  // the reservation holds the FP64 form's digit rows
+  size_t chol_cap = 0;  // and this much Cholesky scratch
 };
 
 std::string key_of(const cov_request& r) {
@@ -169,7 +170,7 @@ static int run_request(cov_server* s, Rec& q, Resident* res, cudaStream_t stream
     // the FP64 form's digits only where the reservation holds them
     if (!q.digits) res->h->sl_rows = res->h->sl_tri = -1;
     const size_t M = (size_t)res->h->M;
-    res->h->chol_scratch_cap = 2 * wl_chol_scratch_est((int64_t)M + 1) + ((size_t)48 << 20);
+    res->h->chol_scratch_cap = q.chol_cap;
     if (cudaMalloc(&res->C, sizeof(double) * M * M) != cudaSuccess ||
         cudaMalloc(&res->D, sizeof(double) * M) != cudaSuccess) {
       cudaGetLastError();
@@ -348,6 +349,16 @@ extern "C" int cov_server_submit(cov_server* s, const cov_request* r, int64_t* i
     q.digits = wl_request_bytes(&r->nz, &r->bins, COV_FP64, s->o.terms, &M, &with, true) == COV_OK &&
                with <= s->o.hbm_budget;
     if (q.digits) q.info.footprint = std::max(q.info.footprint, with);
+  }
+  // the estimate's share of Cholesky scratch; above ~24000 rows it holds single panels
+  // only (M = 24400: 273 ms against 158), so the wide form where the budget holds it
+  q.chol_cap = 2 * wl_chol_scratch_est(q.info.M + 1) + ((size_t)48 << 20);
+  if (s->o.dry_run_us <= 0 && wl_fx_bytes(q.info.M, 2) > q.chol_cap) {
+    const size_t wide = wl_fx_bytes(q.info.M, 8), more = wide > q.chol_cap ? wide - q.chol_cap : 0;
+    if (q.info.footprint + more <= s->o.hbm_budget) {
+      q.info.footprint += more;
+      q.chol_cap += more;
+    }
   }
   if (q.info.footprint > s->o.hbm_budget) {
     q.info.state = COV_REQ_REJECTED;
