@@ -298,7 +298,6 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_sh;
   const int q = warp & 3, half = (warp - 2) >> 2;  // epilogue warp: TMEM lanes 32 q .., columns 16 half .. of a group
-  const int row = q * 32 + lane;
 
   if (warp == 0 && lane == 0) {
     int it = 0;

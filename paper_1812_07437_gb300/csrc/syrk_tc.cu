@@ -405,14 +405,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-__device__ __forceinline__ void tri_tile_tc(int64_t id, int64_t* ti, int64_t* tj) {
-  int64_t i = (int64_t)((sqrt(8.0 * (double)id + 1.0) - 1.0) * 0.5);
-  while (i * (i + 1) / 2 > id) --i;
-  while ((i + 1) * (i + 2) / 2 <= id) ++i;
-  *ti = i;
-  *tj = id - i * (i + 1) / 2;
-}
-
 // ---------------------------------------------------------------- 256 x 256 tiles
 // One CTA per 256 x 256 lower tile: rows I0..I0+255 against rows J0..J0+255.
 // Two TMEM accumulators of 128 x 256 FP32 (all 512 columns), D_h for the row
