@@ -37,10 +37,12 @@ struct SlShape {  // NG groups of 32 columns
   static constexpr int kSmem = SL_STAGES * kStage + 1024;
 };
 
-// X = RN(x 2^55) (ties to even) for |x| < 4, by integer operations on the bits of x
+// X = RN(x 2^55) (ties to even) for |x| < 4, by integer operations on the bits of x; 0 for
+// an infinity or NaN, which no digit holds (its row is marked, see k_sl_norm)
 __device__ __forceinline__ long long sl_int(double x) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const int E = (int)((b >> 52) & 0x7FFu);
+  if (E == 0x7FF) return 0;
   const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);  // (subnormals round to 0 either way)
   const int sh = 1020 - E;  // X = RN(m / 2^sh); sh >= -3
   unsigned long long q;

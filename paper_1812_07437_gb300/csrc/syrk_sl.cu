@@ -107,8 +107,17 @@ struct SlSsc {
   const double *wchi, *sigw2, *chi, *RP3, *RB3;
 };
 
+// Exponent of a row that is not finite (an FP64 row's is below 1100 in magnitude): all
+// elements of its row and column are NaN.
+#define SL_BAD (1 << 20)
+__device__ __forceinline__ double sl_value(unsigned long long sum, int ei, int ej) {
+  const int e = ei + ej - 62;
+  return e > SL_BAD / 2 ? __longlong_as_double(0x7FF8000000000000ll) : scaled_to_double_rn((long long)sum, e);
+}
+
 // One warp per row: its lensing weight and super-sample entry at every node, scaled by
-// the row's power of two (exponent in rexp).
+// the row's power of two (exponent in rexp; SL_BAD where the row holds an infinity or NaN
+// or its norm overflows).
 __global__ void __launch_bounds__(256) k_sl_norm(SlSig g, int64_t rows, const int32_t* __restrict__ rd,
                                                  const double* __restrict__ W, double wscale,
                                                  const double* __restrict__ s2, SlSsc ss, double* wrow, double* srow,
@@ -138,14 +147,15 @@ __global__ void __launch_bounds__(256) k_sl_norm(SlSig g, int64_t rows, const in
     acc = fma(w * w, sq[n], acc);
   }
   acc = warp_sum(acc);
+  const bool bad = !isfinite(acc);
   int e = 0;
-  if (acc > 0.0) frexp(sqrt(acc) * (0.70710678118654752440 * (1.0 + 1e-9)), &e);
-  const double sc = ldexp(1.0, -e);
+  if (!bad && acc > 0.0) frexp(sqrt(acc) * (0.70710678118654752440 * (1.0 + 1e-9)), &e);
+  const double sc = bad ? 0.0 : ldexp(1.0, -e);  // (NaN and infinity stay what they are or become NaN: digits of 0)
   for (int n = lane; n < nchi; n += 32) {
     wo[n] *= sc;
     if (ss.nssc) so[n] *= sc;
   }
-  if (lane == 0) rexp[a] = e;
+  if (lane == 0) rexp[a] = bad ? SL_BAD : e;
 }
 
 // Digits of 128 rows x 32 K, one contiguous 56 KB block per (row block, K block):
@@ -320,7 +330,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
         const unsigned long long off = SL_BIAS * (unsigned long long)(kb1 - kb0);
         const int64_t gr = ti * SL_BM + sl_row<false>(q, lane, 0);
         if (gr < A.row1) {
-          const int er = A.rexp[gr] - 62;
+          const int er = A.rexp[gr];
           double* p = A.out.at(gr, tj * SL_BM);
 #pragma unroll
           for (int j = 0; j < SL_NG; ++j)
@@ -328,7 +338,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
             for (int c = 0; c < 16; ++c) {
               const int lc = sl_col<false>(half, lane, j, c);
               const int64_t gc = tj * SL_BM + lc;
-              if (gc <= gr) p[lc] = scaled_to_double_rn((long long)(acc[j][c] - off), er + __ldg(A.rexp + gc));
+              if (gc <= gr) p[lc] = sl_value(acc[j][c] - off, er, __ldg(A.rexp + gc));
             }
         }
       } else {
@@ -358,7 +368,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
         const int lr = e & (SL_BM - 1), lc = e >> 7;
         const int64_t gr = ti * SL_BM + lr, gc = tj * SL_BM + lc;
         if (gr < A.row1 && gc <= gr)
-          *A.out.at(gr, gc) = scaled_to_double_rn((long long)(__ldcg(p + e) - off), A.rexp[gr] + A.rexp[gc] - 62);
+          *A.out.at(gr, gc) = sl_value(__ldcg(p + e) - off, A.rexp[gr], A.rexp[gc]);
       }
     }
   }
