@@ -199,7 +199,14 @@ int cov_spectra(cov_handle* h, double* d_D, void* stream);
  * M x M, leading dimension ldc) as the sum of the selected terms.
  * precision selects the arithmetic of the 1-halo (chi, M) contraction
  * (COV_FP64 or COV_SPLIT_BF16); every other term is FP64.  Requires a
- * preceding cov_spectra on the same handle. */
+ * preceding cov_spectra on the same handle.
+ *
+ * COV_FP64 is ordered on the stream and returns without waiting for it; after
+ * a first call with the same terms it can be captured into a graph.  Where a
+ * bounded device wait of its contraction expires, the elements left incomplete
+ * are NaN, and the next cov_snr, cov_snr_tiles, cov_pca or cov_batch_snr on
+ * the handle returns COV_ERR_TIMEOUT.  COV_SPLIT_BF16 synchronises the stream
+ * and returns COV_ERR_TIMEOUT itself. */
 int cov_assemble(cov_handle* h, double* d_C, int64_t ldc, unsigned terms, int precision, void* stream);
 
 /* Output layouts of cov_assemble_band. */
@@ -218,8 +225,8 @@ int cov_assemble(cov_handle* h, double* d_C, int64_t ldc, unsigned terms, int pr
  *   With row0 = 0 and nrows = M this is the whole lower-packed matrix.
  * Tile entries above the diagonal and below row M are not written.
  * row0 must be a multiple of 256 and row0 + nrows a multiple of 256 or M.
- * precision: COV_SPLIT_BF16 or COV_FP64 as in cov_assemble; COV_TERM_SSC
- * requires COV_TERM_1H.  The operands (factor rows, trispectrum table) are
+ * precision: COV_SPLIT_BF16 or COV_FP64 as in cov_assemble (also for what each
+ * waits for and reports); COV_TERM_SSC requires COV_TERM_1H.  The operands (factor rows, trispectrum table) are
  * built by the first band after cov_spectra (or a change of terms or
  * precision) and reused by the following bands; a band computes exactly what
  * cov_assemble computes for its rows.  Requires a preceding cov_spectra. */

@@ -240,7 +240,7 @@ static void free_all(cov_handle* h) {
                   h->B1hp,  h->Bp,    h->A,       h->Ahi,     h->Alo,    h->Ascale, h->G2,        h->G3,
                   h->C2,    h->C3,    h->tc_status, h->Thi,   h->Tlo,    h->Tscale, h->Trows,     h->Tmat,
                   h->Srows, h->cosmo_d, h->Fsig,  h->Esig,    h->Msig,   h->FsigT,  h->EsigT,     h->MsigT,
-                  h->invN,  h->omN,   h->work,    h->chol_scratch, h->chol_status, h->mb, h->omb, h->cs,
+                  h->invN,  h->omN,   h->work,    h->chol_scratch, h->piv_status, h->mb, h->omb, h->cs,
                   h->cw,    h->sigF,  h->ac,      h->bmask,   h->gblk,   h->wait_flag, h->pca_buf,
                   h->kap,   h->kgram, h->kcol,    h->kn,      h->koff,      h->plist,
                   h->knode, h->kwt,   h->kw8,     h->kws,     h->zsrc,      h->gsel,    h->cmass,   h->chebm,
@@ -256,7 +256,6 @@ static void free_all(cov_handle* h) {
     if (z.cnt) cudaFree(z.cnt);
     if (z.out) cudaFree(z.out);
   }
-  if (h->piv_status) cudaFree(h->piv_status);
   if (h->batch_C) cudaFree(h->batch_C);
   if (h->batch_D) cudaFree(h->batch_D);
 }

@@ -445,8 +445,8 @@ static int gauss(cov_handle* h, const GatherArgs& g, int64_t r0, int64_t r1, Out
 // The 1-halo trispectrum table T = R R^T of the PT term (Eq. CovBB): digit rows and
 // the exact-sum contraction (FP64 form; FP64 rows and an FP64 product where the
 // digits do not fit), or BF16 hi/lo rows built straight from the bin pair
-// signatures and the tensor-core contraction.  The FP64 form's caller resets and
-// checks the status word.
+// signatures and the tensor-core contraction.  The FP64 form's caller resets the
+// status word.
 static int build_ttable(cov_handle* h, int precision, cudaStream_t s) {
   int rc;
   const int64_t K = h->K;
@@ -563,8 +563,6 @@ int wl_assemble(cov_handle* h, double* C, int64_t ldc, unsigned terms, int preci
       return rc;
     wl_stage_end(h, tk, s);
   }
-  if (fp64 && (h->sl_rows > 0 || h->sl_tri > 0) && (terms & (COV_TERM_1H | COV_TERM_BBPT)))
-    return wl_tc_status_check(h, s);
   return COV_OK;
 }
 
@@ -716,7 +714,5 @@ int wl_assemble_band(cov_handle* h, int64_t row0, int64_t nrows, OutMap out, uns
     if ((rc = gemm_lower_band(h, h->Srows, h->nchi, row1, h->nchi, 1.0, out, s))) return rc;
     wl_stage_end(h, tk, s);
   }
-  if (precision == COV_FP64 && (digits || h->sl_tri > 0) && (terms & (COV_TERM_1H | COV_TERM_BBPT)))
-    return wl_tc_status_check(h, s);
   return COV_OK;
 }

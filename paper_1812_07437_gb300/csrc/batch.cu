@@ -125,7 +125,7 @@ int eager_step(cov_handle* h, unsigned terms, int precision, double* C, double* 
       if ((rc = wl_snr(h, C, h->M, D, w, snr3 + (size_t)w * h->nl, s))) return rc;
     return COV_OK;
   }
-  for (int* w : {h->chol_status, h->piv_status}) WL_CHECK(h, cudaMemsetAsync(w, 0, sizeof(int), s));
+  WL_CHECK(h, cudaMemsetAsync(h->piv_status, 0, 2 * sizeof(int), s));
   h->deferred = true;
   rc = snr_three(h, lane, s);
   h->deferred = false;
@@ -335,9 +335,8 @@ extern "C" int cov_batch_snr(cov_handle* h, const cov_cosmology* cosmos, int n, 
     cudaError_t ce = cudaHostAlloc(&po.p, sizeof(double) * per * n, cudaHostAllocDefault);
     if (ce != cudaSuccess) return wl_cuda(h, ce, "cudaHostAlloc (batch staging)");
     double* out = (double*)po.p;
-    int* words[3] = {h->tc_status, h->chol_status, h->piv_status};  // the first is unused by the FP64 form
-    for (int* w : words)
-      if (w) WL_CHECK(h, cudaMemsetAsync(w, 0, sizeof(int), s));
+    if (h->tc_status) WL_CHECK(h, cudaMemsetAsync(h->tc_status, 0, sizeof(int), s));
+    WL_CHECK(h, cudaMemsetAsync(h->piv_status, 0, 2 * sizeof(int), s));
     // 2. cosmologies 1..n-1 as one graph launch (a device-side loop)
     bool built = false;
     double cap_ms = 0.0, run_ms = 0.0;
@@ -397,12 +396,11 @@ extern "C" int cov_batch_snr(cov_handle* h, const cov_cosmology* cosmos, int n, 
       cudaGraphExecDestroy(exec);
       if (ce != cudaSuccess) return wl_cuda(h, ce, "batch replays");
     }
-    int st[3] = {0, 0, 0};
-    for (int w = 0; w < 3; ++w)
-      if (words[w]) WL_CHECK(h, cudaMemcpyAsync(&st[w], words[w], sizeof(int), cudaMemcpyDeviceToHost, s));
-    WL_CHECK(h, cudaStreamSynchronize(s));
-    if (st[0] || st[1]) return wl_fail(h, COV_ERR_TIMEOUT, "batch: a bounded mbarrier wait expired");
-    if (st[2]) return wl_fail(h, COV_ERR_NOT_PD, "batch: a Cholesky met a non-positive pivot");
+    int tc = 0;
+    if (h->tc_status) WL_CHECK(h, cudaMemcpyAsync(&tc, h->tc_status, sizeof(int), cudaMemcpyDeviceToHost, s));
+    rc = wl_snr_status(h, s);
+    if (tc) return wl_fail(h, COV_ERR_TIMEOUT, "batch: a bounded mbarrier wait expired");
+    if (rc) return rc;
     // S/N of a selection with no rows stays NaN (the eager step wrote the host copy)
     for (int k = 1; k < n; ++k) {
       double* o = out + per * k;

@@ -136,11 +136,8 @@ __global__ void k_snr_prefix(int64_t Ms, OutMap W, const int64_t* cnt, int nl, d
 static int factor_and_prefix(cov_handle* h, OutMap Wm, int64_t Ms, const int* perm, const double* C, int64_t ldc,
                              const double* D, const int64_t* cnt_d, double* out_d, double* h_snr, cudaStream_t s) {
   int rc;
-  if (!h->chol_status) WL_CHECK(h, cudaMalloc(&h->chol_status, sizeof(int)));
-  if (!h->deferred) {
-    WL_CHECK(h, cudaMemsetAsync(h->chol_status, 0, sizeof(int), s));
-    WL_CHECK(h, cudaMemsetAsync(h->piv_status, 0, sizeof(int), s));
-  }
+  if ((rc = wl_status_words(h, s))) return rc;
+  if (!h->deferred) WL_CHECK(h, cudaMemsetAsync(h->piv_status, 0, 2 * sizeof(int), s));
   if ((rc = wl_fx_factor(h, Wm, Ms, perm, C, ldc, D, s))) return rc;
   int tk = wl_stage_begin(h, ST_SNR_PREFIX, s);
   k_snr_prefix<<<h->nl, 256, 0, s>>>(Ms, Wm, cnt_d, h->nl, out_d);
@@ -151,14 +148,27 @@ static int factor_and_prefix(cov_handle* h, OutMap Wm, int64_t Ms, const int* pe
   return wl_snr_status(h, s);
 }
 
-// The status words of the factorisations on s (synchronises it)
+int wl_status_words(cov_handle* h, cudaStream_t s) {
+  if (h->piv_status) return COV_OK;
+  WL_CHECK(h, cudaMalloc(&h->piv_status, 3 * sizeof(int)));
+  h->chol_status = h->piv_status + 1;
+  h->sl_report = h->piv_status + 2;
+  WL_CHECK(h, cudaMemsetAsync(h->piv_status, 0, 3 * sizeof(int), s));
+  return COV_OK;
+}
+
+// The status words of the factorisations on s, and of the FP64 assemblies before them,
+// which do not wait for their kernels themselves (synchronises s)
 int wl_snr_status(cov_handle* h, cudaStream_t s) {
-  int status = 0, tstatus = 0;
-  WL_CHECK(h, cudaMemcpyAsync(&status, h->piv_status, sizeof(int), cudaMemcpyDeviceToHost, s));
-  WL_CHECK(h, cudaMemcpyAsync(&tstatus, h->chol_status, sizeof(int), cudaMemcpyDeviceToHost, s));
+  int w[3] = {0, 0, 0};
+  WL_CHECK(h, cudaMemcpyAsync(w, h->piv_status, sizeof(w), cudaMemcpyDeviceToHost, s));
   WL_CHECK(h, cudaStreamSynchronize(s));
-  if (tstatus) return wl_fail(h, COV_ERR_TIMEOUT, "Cholesky trailing update: a bounded mbarrier wait expired");
-  if (status) return wl_fail(h, COV_ERR_NOT_PD, "Cholesky met a non-positive pivot");
+  if (w[2]) {
+    WL_CHECK(h, cudaMemsetAsync(h->sl_report, 0, sizeof(int), s));
+    return wl_fail(h, COV_ERR_TIMEOUT, "FP64 contraction of an earlier assembly: a bounded mbarrier wait expired");
+  }
+  if (w[1]) return wl_fail(h, COV_ERR_TIMEOUT, "Cholesky trailing update: a bounded mbarrier wait expired");
+  if (w[0]) return wl_fail(h, COV_ERR_NOT_PD, "Cholesky met a non-positive pivot");
   return COV_OK;
 }
 
@@ -192,10 +202,6 @@ static int selection(cov_handle* h, int slot, cudaStream_t s) {
     WL_CHECK(h, cudaMalloc(&z.out, sizeof(double) * h->nl));
     h->allocated += sizeof(int) * (size_t)std::max<int64_t>(Ms, 1) + sizeof(int64_t) * h->nl + sizeof(double) * h->nl;
   }
-  if (!h->piv_status) {
-    WL_CHECK(h, cudaMalloc(&h->piv_status, sizeof(int)));
-    WL_CHECK(h, cudaMemsetAsync(h->piv_status, 0, sizeof(int), s));
-  }
   if (Ms) WL_CHECK(h, cudaMemcpyAsync(z.perm, sel.data(), sizeof(int) * Ms, cudaMemcpyHostToDevice, s));
   WL_CHECK(h, cudaMemcpyAsync(z.cnt, cnt.data(), sizeof(int64_t) * h->nl, cudaMemcpyHostToDevice, s));
   WL_CHECK(h, cudaStreamSynchronize(s));  // sel and cnt are host memory read by the copies
@@ -209,8 +215,7 @@ int wl_snr_prepare(cov_handle* h, cudaStream_t s) {
   int rc;
   for (int w = 0; w < 3; ++w)
     if ((rc = selection(h, w, s))) return rc;
-  if (!h->chol_status) WL_CHECK(h, cudaMalloc(&h->chol_status, sizeof(int)));
-  return COV_OK;
+  return wl_status_words(h, s);
 }
 
 // perm: another order of the selection's rows (the factor is then of that order, and the

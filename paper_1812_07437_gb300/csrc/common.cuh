@@ -230,7 +230,10 @@ struct cov_handle {
   size_t chol_scratch_cap = 0;   // bytes it should stay within (the server's reservation; 0: no limit)
   cudaStream_t side = nullptr;   // look-ahead stream of the Cholesky panel kernels
   cudaEvent_t ev_cols = nullptr, ev_panel = nullptr;
-  int* chol_status = nullptr;
+  // status words, one allocation (wl_status_words): a non-positive pivot seen, an expired wait in a
+  // Cholesky update (both sticky inside a batch), an expired wait in an FP64 contraction since the
+  // last call that read the words
+  int *piv_status = nullptr, *chol_status = nullptr, *sl_report = nullptr;
   bool spectra_ready = false;
   int row_set = 0, row_order = 0;  // COV_ROWS_*, COV_ORDER_*
   cov_cosmology* cosmo_d = nullptr;  // the cosmology the kernels read (device copy of cosmo)
@@ -246,7 +249,6 @@ struct cov_handle {
     int64_t* cnt = nullptr;
     double* out = nullptr;
   } sel[4];
-  int* piv_status = nullptr;  // non-positive pivot seen (sticky inside a batch)
   double *batch_C = nullptr, *batch_D = nullptr;  // covariance and data vector of cov_batch_snr
   cudaStream_t batch_stream = nullptr;             // cov_batch_snr runs (and captures) on this stream
   cudaEvent_t batch_ev = nullptr;
@@ -291,7 +293,8 @@ int wl_snr_tiles(cov_handle* h, double* Ct, const double* D, double* h_snr, cuda
 int wl_assemble_band(cov_handle* h, int64_t row0, int64_t nrows, OutMap out, unsigned terms, int precision,
                      cudaStream_t s);
 int wl_snr_prepare(cov_handle* h, cudaStream_t s);  // chol.cu
-int wl_snr_status(cov_handle* h, cudaStream_t s);   // chol.cu
+int wl_status_words(cov_handle* h, cudaStream_t s);  // chol.cu
+int wl_snr_status(cov_handle* h, cudaStream_t s);    // chol.cu
 int wl_snr(cov_handle* h, const double* d_C, int64_t ldc, const double* d_D, int which, double* h_snr,
            cudaStream_t s, const int* perm = nullptr);  // chol.cu
 int wl_gemm_lower_fp64(cov_handle* h, const double* A, int64_t lda, const double* B, int64_t ldb, double* C,

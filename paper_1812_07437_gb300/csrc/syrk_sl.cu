@@ -276,9 +276,9 @@ struct SlArgs {
   int nk, ns;                 // K blocks; CTAs that share a tile's K range
   const int* rexp;
   OutMap out;
-  int* status;
+  int *status, *report;       // an expired wait of this assembly; of any since the host last read it
   unsigned long long* part;   // [tile][column][row] exact partial sums (ns > 1), zero at launch
-  int* ticket;                // [tile] CTAs that have delivered (ns > 1), zero at launch
+  int* ticket;                // [tile] CTAs that have delivered (ns > 1), 2^16 for each that gave up, zero at launch
 };
 
 // One CTA per (128 x 128 lower tile, K range).  Warp 0 loads (TMA, two stages of a K
@@ -287,13 +287,14 @@ struct SlArgs {
 // columns each), eight warps recombine the set of the group before in registers (64
 // 64-bit sums per thread).  Where a launch has too few tiles for the SMs, ns CTAs take
 // parts of a tile's K range, add their 64-bit sums atomically (integers: any order
-// gives the same value) and the last one converts.
+// gives the same value) and the last one converts.  The host does not wait for this kernel:
+// where a wait expires, the elements that it leaves incomplete are stored as NaN.
 __global__ void __launch_bounds__(SL_THREADS, 1)
     k_syrk_sl(const __grid_constant__ CUtensorMap map_i, const __grid_constant__ CUtensorMap map_j, SlArgs A) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) SlBars bars;
   __shared__ uint32_t tmem_sh;
-  __shared__ int last_sh;
+  __shared__ int last_sh, gave_up;
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t tile = blockIdx.x / A.ns;
@@ -301,7 +302,10 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
   const int kb0 = (int)((int64_t)A.nk * sp / A.ns), kb1 = (int)((int64_t)A.nk * (sp + 1) / A.ns);
   int64_t ti, tj;
   sl_tile(tile, A.t0, A.t1, &ti, &tj);
-  if (threadIdx.x == 0) sl_bars_init(&bars);
+  if (threadIdx.x == 0) {
+    sl_bars_init(&bars);
+    gave_up = 0;
+  }
   if (warp == 0) sl_tmem_alloc(&tmem_sh);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -325,30 +329,29 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
     int it = 0;
     sl_drain_init<false>(&bars, tmem, q, half, lane);
     const bool ok = sl_drain<SL_NG, false>(acc, &bars, tmem, q, half, lane, kb1 - kb0, it, A.status);
-    if (ok && *(volatile int*)A.status == 0) {
-      if (A.ns == 1) {
-        const unsigned long long off = SL_BIAS * (unsigned long long)(kb1 - kb0);
-        const int64_t gr = ti * SL_BM + sl_row<false>(q, lane, 0);
-        if (gr < A.row1) {
-          const int er = A.rexp[gr];
-          double* p = A.out.at(gr, tj * SL_BM);
-#pragma unroll
-          for (int j = 0; j < SL_NG; ++j)
-#pragma unroll
-            for (int c = 0; c < 16; ++c) {
-              const int lc = sl_col<false>(half, lane, j, c);
-              const int64_t gc = tj * SL_BM + lc;
-              if (gc <= gr) p[lc] = sl_value(acc[j][c] - off, er, __ldg(A.rexp + gc));
-            }
-        }
-      } else {
-        unsigned long long* p = A.part + (size_t)tile * (SL_BM * SL_BM);
+    if (!ok) gave_up = 1;
+    if (A.ns == 1) {
+      const unsigned long long off = SL_BIAS * (unsigned long long)(kb1 - kb0);
+      const int64_t gr = ti * SL_BM + sl_row<false>(q, lane, 0);
+      if (gr < A.row1) {
+        const int er = ok ? A.rexp[gr] : SL_BAD;
+        double* p = A.out.at(gr, tj * SL_BM);
 #pragma unroll
         for (int j = 0; j < SL_NG; ++j)
 #pragma unroll
-          for (int c = 0; c < 16; ++c)
-            atomicAdd(p + (size_t)sl_col<false>(half, lane, j, c) * SL_BM + sl_row<false>(q, lane, c), acc[j][c]);
+          for (int c = 0; c < 16; ++c) {
+            const int lc = sl_col<false>(half, lane, j, c);
+            const int64_t gc = tj * SL_BM + lc;
+            if (gc <= gr) p[lc] = sl_value(acc[j][c] - off, er, __ldg(A.rexp + gc));
+          }
       }
+    } else if (ok) {
+      unsigned long long* p = A.part + (size_t)tile * (SL_BM * SL_BM);
+#pragma unroll
+      for (int j = 0; j < SL_NG; ++j)
+#pragma unroll
+        for (int c = 0; c < 16; ++c)
+          atomicAdd(p + (size_t)sl_col<false>(half, lane, j, c) * SL_BM + sl_row<false>(q, lane, c), acc[j][c]);
     }
   }
   __syncwarp();
@@ -357,10 +360,14 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
   if (A.ns > 1) __threadfence();
   __syncthreads();
   if (warp == 0) sl_tmem_free(tmem);
+  if (threadIdx.x == 0 && *(volatile int*)A.status != 0) atomicExch(A.report, 1);
   if (A.ns > 1) {
-    if (threadIdx.x == 0) last_sh = atomicAdd(A.ticket + tile, 1) == A.ns - 1;
+    if (threadIdx.x == 0) {  // 1: the last CTA of the tile, 2: and one of them gave up
+      const int add = gave_up ? 65537 : 1, t = atomicAdd(A.ticket + tile, add) + add;
+      last_sh = (t & 65535) != A.ns ? 0 : t > 65535 ? 2 : 1;
+    }
     __syncthreads();
-    if (last_sh && *(volatile int*)A.status == 0) {
+    if (last_sh) {
       __threadfence();
       const unsigned long long off = SL_BIAS * (unsigned long long)A.nk;
       const unsigned long long* p = A.part + (size_t)tile * (SL_BM * SL_BM);
@@ -368,7 +375,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
         const int lr = e & (SL_BM - 1), lc = e >> 7;
         const int64_t gr = ti * SL_BM + lr, gc = tj * SL_BM + lc;
         if (gr < A.row1 && gc <= gr)
-          *A.out.at(gr, gc) = sl_value(__ldcg(p + e) - off, A.rexp[gr], A.rexp[gc]);
+          *A.out.at(gr, gc) = sl_value(__ldcg(p + e) - off, last_sh == 2 ? SL_BAD : A.rexp[gr], A.rexp[gc]);
       }
     }
   }
@@ -494,7 +501,8 @@ int wl_sl_alloc(cov_handle* h, bool tri, bool* use, cudaStream_t s) {
 }
 
 // Lower part of rows [out.row0, row1) of the contraction (tri: the trispectrum table)
-// into out: the first writer.  The status word is reset and checked by the caller.
+// into out: the first writer.  The caller resets the status word; what the launch reports is
+// read by the next call that waits for the device (wl_snr_status).
 int wl_sl_syrk(cov_handle* h, bool tri, int nssc, OutMap out, int64_t row1, cudaStream_t s) {
   const int64_t rows = tri ? h->ntrow : h->M;
   const int64_t nb = (rows + SL_BM - 1) / SL_BM, nk = sl_nk((int64_t)h->K + nssc);
@@ -503,6 +511,7 @@ int wl_sl_syrk(cov_handle* h, bool tri, int nssc, OutMap out, int64_t row1, cuda
   if (ntiles <= 0) return COV_OK;
   CUtensorMap mi, mj;
   int rc;
+  if ((rc = wl_status_words(h, s))) return rc;
   uint8_t* sl = tri ? h->Tsl : h->Asl;
   if ((rc = wl_sl_map(h, &mi, sl, nb * nk, SL_BM)) || (rc = wl_sl_map(h, &mj, sl, nb * nk, SL_BN))) return rc;
   // CTAs per tile: with one per SM, the parts (of at least 16 K blocks) that finish in
@@ -521,7 +530,8 @@ int wl_sl_syrk(cov_handle* h, bool tri, int nssc, OutMap out, int64_t row1, cuda
       }
     }
   }
-  SlArgs a{rows, row1, t0, t1, (int)nk, ns, tri ? h->Texp : h->Aexp, out, h->tc_status, h->sl_part, nullptr};
+  SlArgs a{rows, row1, t0, t1, (int)nk, ns, tri ? h->Texp : h->Aexp, out, h->tc_status, h->sl_report,
+           h->sl_part, nullptr};
   a.ticket = (int*)(h->sl_part + (size_t)SL_SPLIT_TILES * SL_BM * SL_BM);
   if (ns > 1) {
     WL_CHECK(h, cudaMemsetAsync(h->sl_part, 0, (size_t)ntiles * SL_BM * SL_BM * 8, s));
