@@ -559,7 +559,9 @@ extern "C" int cov_assemble_band(cov_handle* h, int64_t row0, int64_t nrows, dou
     return wl_fail(h, COV_ERR_INVALID, "cov_assemble_band: ldc below row0 + nrows");
   if (!h->spectra_ready) return wl_fail(h, COV_ERR_INVALID, "cov_spectra must run before cov_assemble_band");
   OutMap out = layout == COV_LAYOUT_TILES ? out_tiles(d_C, row0) : out_rows(d_C, ldc, row0);
-  return wl_assemble_band(h, row0, nrows, out, terms, precision, (cudaStream_t)stream);
+  const int rc = wl_assemble_band(h, row0, nrows, out, terms, precision, (cudaStream_t)stream);
+  if (rc) h->ops_terms = -1;  // a retry prepares its operands again
+  return rc;
 }
 
 extern "C" int cov_snr_tiles(cov_handle* h, double* d_Ct, const double* d_D, double* h_snr, void* stream) {

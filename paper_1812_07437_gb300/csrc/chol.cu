@@ -164,6 +164,7 @@ int wl_snr_status(cov_handle* h, cudaStream_t s) {
   WL_CHECK(h, cudaMemcpyAsync(w, h->piv_status, sizeof(w), cudaMemcpyDeviceToHost, s));
   WL_CHECK(h, cudaStreamSynchronize(s));
   if (w[2]) {
+    h->ops_terms = -1;  // the trispectrum table that a band prepared may be what is incomplete
     WL_CHECK(h, cudaMemsetAsync(h->sl_report, 0, sizeof(int), s));
     return wl_fail(h, COV_ERR_TIMEOUT, "FP64 contraction of an earlier assembly: a bounded mbarrier wait expired");
   }

@@ -22,6 +22,9 @@ extern "C" int report(cov_handle* h) {  // as k_syrk_sl does when a wait of its 
   const int one = 1;
   return (int)cudaMemcpy(h->sl_report, &one, sizeof(int), cudaMemcpyHostToDevice);
 }
+extern "C" int spoil_table(cov_handle* h) {  // a trispectrum table whose tiles were left incomplete
+  return (int)cudaMemset(h->Tmat, 0xFF, sizeof(double) * h->ntrow * h->ntrow);
+}
 """
 
 
@@ -104,4 +107,24 @@ def test_expired_wait_is_reported_by_the_next_synchronising_call(poke):
             call()
         assert e.value.code == N.COV_ERR_TIMEOUT and "earlier assembly" in str(e.value)
         assert np.array_equal(h.snr(C, D), ref)  # reported once
+    h.close()
+
+
+def test_a_reported_wait_makes_the_next_band_prepare_its_operands(poke):
+    h = _handle()
+    C = torch.zeros((h.M, h.M), dtype=torch.float64, device="cuda")
+    D = torch.zeros(h.M, dtype=torch.float64, device="cuda")
+    h.spectra(D)
+    _call(h, C, True, N.COV_TERMS_ALL)
+    torch.cuda.synchronize()
+    ref = C.clone()
+    assert poke.spoil_table(h.h) == 0 and poke.report(h.h) == 0
+    _call(h, C, True, N.COV_TERMS_ALL)  # the operands of the first band, the spoilt table among them
+    with pytest.raises(N.CovError) as e:
+        h.snr(C, D)
+    assert e.value.code == N.COV_ERR_TIMEOUT
+    assert not torch.equal(C, ref)
+    _call(h, C, True, N.COV_TERMS_ALL)
+    torch.cuda.synchronize()
+    assert torch.equal(C, ref)
     h.close()
