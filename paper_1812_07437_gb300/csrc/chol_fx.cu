@@ -612,8 +612,11 @@ size_t wl_fx_bytes(int64_t n, int w) {
 
 // The scratch, grown on demand: super-panels of four panels (eight for matrices whose
 // trailing update bounds the factorisation: half the passes over the entries), fewer
-// where the memory (or the server's reservation) does not hold them.
-static int fx_scratch(cov_handle* h, int64_t n, int* w_out) {
+// where the memory (or the server's reservation) does not hold them.  A captured step
+// keeps to what the eager one before it allocated.
+static int fx_scratch(cov_handle* h, int64_t n, int* w_out, cudaStream_t s) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (h->deferred) WL_CHECK(h, cudaStreamIsCapturing(s, &cap));
   for (int w = n >= FX_WIDE ? 8 : 4; w >= 1; w >>= 1) {
     const size_t need = wl_fx_bytes(n, w);
     if (w > 1 && h->chol_scratch_cap && need > h->chol_scratch_cap) continue;
@@ -621,13 +624,19 @@ static int fx_scratch(cov_handle* h, int64_t n, int* w_out) {
       *w_out = w;
       return COV_OK;
     }
+    if (cap != cudaStreamCaptureStatusNone) continue;
     if (w > 1) {
-      if (h->deferred && h->chol_scratch) continue;  // (a captured step keeps to what the eager one allocated)
       size_t fr = 0, tot = 0;
       const bool known = cudaMemGetInfo(&fr, &tot) == cudaSuccess;
       if (!known || need > fr / 16 ||
           (h->budget && h->allocated - h->chol_scratch_n + need + ((size_t)64 << 20) > h->budget))
         continue;
+    }
+    if (h->chol_scratch) {  // given back first: never the old and the new buffer at the same time
+      cudaFree(h->chol_scratch);
+      h->allocated -= h->chol_scratch_n;
+      h->chol_scratch = nullptr;
+      h->chol_scratch_n = 0;
     }
     void* p = nullptr;
     cudaError_t e = cudaMalloc(&p, need);
@@ -636,17 +645,13 @@ static int fx_scratch(cov_handle* h, int64_t n, int* w_out) {
       if (w > 1) continue;
       return wl_cuda(h, e, "cudaMalloc (Cholesky scratch)");
     }
-    if (h->chol_scratch) {
-      cudaFree(h->chol_scratch);
-      h->allocated -= h->chol_scratch_n;
-    }
     h->chol_scratch = p;
     h->chol_scratch_n = need;
     h->allocated += need;
     *w_out = w;
     return COV_OK;
   }
-  return COV_OK;
+  return wl_fail(h, COV_ERR_INVALID, "Cholesky scratch not allocated before stream capture");
 }
 
 // Whether `extra` bytes more are beyond the handle's budget.  The Cholesky's scratch is
@@ -714,7 +719,7 @@ int wl_fx_factor(cov_handle* h, OutMap W, int64_t Ms, const int* perm, const dou
   if (h->chol_kernel != 1 && !fx_wide(W))
     return wl_fail(h, COV_ERR_CUDA, "Cholesky: the matrix is not 16-byte aligned");
   if ((rc = fx_attributes(h))) return rc;
-  if ((rc = fx_scratch(h, Ms, &w))) return rc;
+  if ((rc = fx_scratch(h, Ms, &w, s))) return rc;
   if ((rc = wl_side_stream(h))) return rc;
   const int64_t nb = (Ms + SL_BM - 1) / SL_BM;
   const int nkb = 2 * w;
