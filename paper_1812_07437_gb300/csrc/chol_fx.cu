@@ -89,13 +89,14 @@ __device__ __forceinline__ void fx_st2(double* p, unsigned long long a, unsigned
 }
 
 // ---------------------------------------------------------------- scaling
-// rs[i] = C_ii^-1/2 of the selected entries (perm null: row i of W, FP64)
+// rs[i] = C_ii^-1/2 of the selected entries (perm null: row i of W, FP64); the scaled diagonal
+// is 1 by construction, so a variance that is no positive number is caught here
 __global__ void k_fx_rs(int64_t Ms, const int* __restrict__ perm, const double* __restrict__ C, int64_t ldc, OutMap W,
                         double* rs, int* status) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= Ms) return;
   const double d = perm ? C[(int64_t)perm[i] * ldc + perm[i]] : *W.at(i, i);
-  if (!(d > 0.0)) atomicExch(status, 1);
+  if (!(d > 0.0 && isfinite(d))) atomicExch(status, 1);
   rs[i] = 1.0 / sqrt(d);
 }
 
