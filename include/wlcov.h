@@ -46,12 +46,18 @@ extern "C" {
 #define COV_TERM_SSC 16u /* super-sample term (Eq. WLSSCflatskyLimber)        */
 #define COV_TERMS_ALL 31u
 
-/* arithmetic of the (chi, M) contractions.  The split form's elements carry
+/* arithmetic of the (chi, M) contractions.  COV_FP64: each element to FP64
+ * rounding of the sum of its own terms' magnitudes (a few 2^-53; terms below
+ * 2^-104 of the product of the two rows' largest entries do not count).  Its
+ * rows are held as digits for the tensor cores where 14 bytes per entry fit in
+ * the budget or the free memory beside all that the handle may still allocate,
+ * decided at its first FP64 assembly; else as FP64, ~40 times slower, the same
+ * to that rounding.  The split form's elements carry
  * an error of ~1e-5 sqrt(C_aa C_bb); a covariance whose unit-diagonal scaling
  * has eigenvalues near that (strongly overlapping tomographic kernels, e.g. no
  * photo-z scatter and several bins) can then lose positive definiteness and
  * the S/N returns COV_ERR_NOT_PD: assemble such covariances in COV_FP64. */
-#define COV_FP64 0       /* FP64 accuracy: exact digit sums (tensor cores)    */
+#define COV_FP64 0       /* FP64 rounding: exact digit sums (tensor cores)    */
 #define COV_SPLIT_BF16 1 /* tcgen05 tensor cores, A = hi + lo in BF16, FP32 acc */
 
 /* selection for the signal-to-noise (Sec. 5, Eq. eq:SN2) */

@@ -246,7 +246,7 @@ static void free_all(cov_handle* h) {
                   h->knode, h->kwt,   h->kw8,     h->kws,     h->zsrc,      h->gsel,    h->cmass,   h->chebm,
                   h->trigeo, h->zint, h->pk,      h->amp_part, h->Draw,     h->chis,    h->cz,      h->rvir,
                   h->hint,  h->qw,    h->proj,    h->ksum,    h->kticket,
-                  h->Asl,   h->Tsl,   h->Aexp,    h->Texp,    h->trd,       h->sl_s2,   h->sl_w,    h->sl_sr,
+                  h->Asl,   h->Tsl,   h->Aexp,    h->Texp,    h->trd,       h->sl_w,    h->sl_sr,
                   h->sl_part};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -371,7 +371,7 @@ int wl_request_bytes(const cov_nz* nz, const cov_bins* bins, int precision, unsi
     b += wl_sl_fixed_bytes(&h);                                  // weights, exponents, shared partial sums
   if (terms & COV_TERM_1H) {
     if (digits)
-      b += wl_sl_bytes((int64_t)M, (int64_t)(K + nchi));         // digits of the factor and SSC rows
+      b += wl_sl_bytes(&h, false);                               // digits of the factor and SSC rows
     else if (precision == COV_FP64)
       b += M * K * 8 + M * nchi * 8;                             // FP64 factor and SSC rows
     else
@@ -381,7 +381,7 @@ int wl_request_bytes(const cov_nz* nz, const cov_bins* bins, int precision, unsi
   if (terms & COV_TERM_BBPT) {
     b += nt * nt * 8;                                            // trispectrum table
     if (digits)
-      b += wl_sl_bytes((int64_t)nt, (int64_t)K);                 // digits of the trispectrum rows
+      b += wl_sl_bytes(&h, true);                                // digits of the trispectrum rows
     else if (precision == COV_FP64)
       b += nt * K * 8;                                           // FP64 trispectrum rows
     else

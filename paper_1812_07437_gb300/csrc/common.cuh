@@ -212,12 +212,12 @@ struct cov_handle {
   uint16_t *Thi = nullptr, *Tlo = nullptr;  // split trispectrum rows (tensor-core form)
   double* Tscale = nullptr;
   double* Srows = nullptr;  // [M][nchi]
-  // FP64 form on the tensor cores: digit blocks and row exponents of the factor rows
+  // FP64 form on the tensor cores: digit blocks (with their exponents) and row exponents of the factor rows
   // and the trispectrum rows, the latter's descriptors, and their builders' tables
   uint8_t *Asl = nullptr, *Tsl = nullptr;
   int *Aexp = nullptr, *Texp = nullptr;
   int32_t* trd = nullptr;
-  double *sl_s2 = nullptr, *sl_w = nullptr, *sl_sr = nullptr;
+  double *sl_w = nullptr, *sl_sr = nullptr;
   unsigned long long* sl_part = nullptr;  // exact partial sums of tiles shared by several CTAs, then their tickets
   int sl_rows = 0, sl_tri = 0;            // 0 undecided, 1 digits, -1 FP64 rows (k_gemm_lower)
   double* work = nullptr;   // Cholesky workspace (M+1) rows
@@ -303,7 +303,7 @@ int wl_gemm_lower_fp64(cov_handle* h, const double* A, int64_t lda, const double
 int wl_syrk_tc(cov_handle* h, int nssc, OutMap out, cudaStream_t s, int64_t row1 = -1);  // syrk_tc.cu
 int wl_syrk_tc_part(cov_handle* h, int nssc, OutMap out, int64_t r0, int64_t r1, cudaStream_t s);
 int wl_num_sms();  // chol_fx.cu: SMs of the current device
-size_t wl_sl_bytes(int64_t rows, int64_t k);                                             // syrk_sl.cu
+size_t wl_sl_bytes(const cov_handle* h, bool tri);                                       // syrk_sl.cu
 size_t wl_sl_fixed_bytes(const cov_handle* h);                                           // syrk_sl.cu
 int wl_sl_alloc(cov_handle* h, bool tri, bool* use, cudaStream_t s);                     // syrk_sl.cu
 int wl_sl_rows(cov_handle* h, bool tri, int nssc, cudaStream_t s);                       // syrk_sl.cu

@@ -10,8 +10,10 @@
 // stacked in shared memory, the accumulators of the seven levels lie side by side in
 // TMEM, and one MMA of digit t against the first 32 (7 - t) stacked rows lands on the
 // levels t..6 (N = 224, 192, ..., 32).  Small-N MMAs would read the 4 KB of the I digit
-// from shared memory for 8 cycles of work each.  The level sums of a K block are then
-// added exactly to one 64-bit integer per element, in units of 2^-62, modulo 2^64.
+// from shared memory for 8 cycles of work each.  The level sums of a K block combine exactly
+// to one 64-bit integer per element, in units of 2^-62, modulo 2^64: the Cholesky's rows
+// share one scale and it adds them as they are; the contraction's K blocks have exponents of
+// their own, and it aligns them first.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -37,14 +39,14 @@ struct SlShape {  // NG groups of 32 columns
   static constexpr int kSmem = SL_STAGES * kStage + 1024;
 };
 
-// X = RN(x 2^55) (ties to even) for |x| < 4, by integer operations on the bits of x; 0 for
-// an infinity or NaN, which no digit holds (its row is marked, see k_sl_norm)
-__device__ __forceinline__ long long sl_int(double x) {
+// X = RN(x 2^(55 - e)) (ties to even) for |x| < 2^(e + 2), by integer operations on the bits
+// of x; 0 for an infinity or NaN, which no digit holds (its K block is marked, see k_sl_rows)
+__device__ __forceinline__ long long sl_int(double x, int e) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const int E = (int)((b >> 52) & 0x7FFu);
   if (E == 0x7FF) return 0;
   const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);  // (subnormals round to 0 either way)
-  const int sh = 1020 - E;  // X = RN(m / 2^sh); sh >= -3
+  const int sh = 1020 - E + e;  // X = RN(m / 2^sh); sh >= -3
   unsigned long long q;
   if (sh <= 0) {
     q = m << -sh;
@@ -216,8 +218,8 @@ __device__ __forceinline__ bool sl_produce(const CUtensorMap* map_i, const CUten
 // descriptors and addresses live in uniform registers (inside a one-lane branch every
 // operand goes through a register move, ~100 cycles per MMA: more than the MMA itself);
 // the 512 allocated columns start at TMEM address 0.  NEG: the I operand is negated (the
-// sums come out as -A B^T).
-template <int NG, bool NEG>
+// sums come out as -A B^T).  LV 8 forms the level t + u = 7 as well (six pairs of digits).
+template <int NG, bool NEG, int LV = SL_S>
 __device__ __forceinline__ bool sl_issue(uint8_t* smem, SlBars* B, int nkb, int& it, int* status) {
   constexpr int STAGE = SlShape<NG>::kStage;
   uint32_t leader;
@@ -237,9 +239,10 @@ __device__ __forceinline__ bool sl_issue(uint8_t* smem, SlBars* B, int nkb, int&
       for (int k = 0; k < SL_BK / 16; ++k)
 #pragma unroll
         for (int t = 0; t < SL_S; ++t) {
-          // BF16 x BF16 -> FP32, K-major, M = 128, N = 32 (7 - t): digit t against the digits 0 .. 6 - t
+          // BF16 x BF16 -> FP32, K-major, M = 128, N = 32 per digit: digit t against the digits 0 .. LV - 1 - t
+          const int nu = LV - t < SL_S ? LV - t : SL_S;
           const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (NEG ? 1u << 13 : 0u) |
-                                 ((uint32_t)((SL_BN * (SL_S - t)) >> 3) << 17) | ((uint32_t)(SL_BM >> 4) << 24);
+                                 ((uint32_t)((SL_BN * nu) >> 3) << 17) | ((uint32_t)(SL_BM >> 4) << 24);
           asm volatile(
               "{\n .reg .pred p, q;\n setp.ne.b32 p, 1, 0;\n setp.ne.b32 q, %4, 0;\n @q "
               "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dt + (uint32_t)(t * SL_BN)),
@@ -270,13 +273,13 @@ __device__ __forceinline__ void sl_issue_end(SlBars* B, int lane) {
    (257ull * SL_MAGIC & 0xFFFFFFFFull))
 
 // Epilogue warps, once per CTA: the starting value into both accumulator sets
-template <bool FRAG>
+template <bool FRAG, int LV = SL_S>
 __device__ __forceinline__ void sl_drain_init(SlBars* B, uint32_t tmem, int q, int half, int lane) {
   const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * 16);
 #pragma unroll
   for (int b = 0; b < 2; ++b) {
 #pragma unroll
-    for (int g = 0; g < SL_S; ++g) {
+    for (int g = 0; g < LV; ++g) {
 #pragma unroll
       for (int h = 0; h < 4; ++h) sl_tmem_st4<FRAG>(tbase + sl_part<FRAG>(h) + (uint32_t)(b * 256 + g * SL_BN), SL_MAGIC);
     }
