@@ -30,6 +30,11 @@
 // FP64 diagonal blocks and panel solves: the joint S/N of M = 6375 14.4 -> 7.9 ms, of
 // M = 818 1.28 -> 0.78 ms, the one in place at M = 24400 268 -> 158 ms.
 //
+// The integers are modulo 2^64, four times the unit diagonal.  In a positive definite matrix
+// nothing leaves [-1, 1]; in another one a row wraps only after its factor entries' squares
+// have added up to more than its diagonal entry, so the panel kernel keeps that sum of every
+// row (FP32) and raises the pivot status beyond FX_NORM.
+//
 // Error: entries 2^-63 by rounding, updates 2^-56 per digit row against the unit
 // diagonal, i.e. below that of an FP64 factorisation (2^-53 per operation).
 #include <algorithm>
@@ -42,6 +47,7 @@
 // eight; no difference at 6375, where the scratch is then smaller)
 #define FX_WIDE 12288
 #define FX_ONE (1ll << 62)
+#define FX_NORM 1.0625f  // (at most 1 up to the FP32 sums' rounding, ~2e-4 at 2800 panels)
 
 // RN(x 2^62) for |x| <= 1 (2^-30 beyond counts as rounding); anything else, NaN
 // included, cannot be an entry of a scaled positive definite matrix: status
@@ -92,12 +98,13 @@ __device__ __forceinline__ void fx_st2(double* p, unsigned long long a, unsigned
 // rs[i] = C_ii^-1/2 of the selected entries (perm null: row i of W, FP64); the scaled diagonal
 // is 1 by construction, so a variance that is no positive number is caught here
 __global__ void k_fx_rs(int64_t Ms, const int* __restrict__ perm, const double* __restrict__ C, int64_t ldc, OutMap W,
-                        double* rs, int* status) {
+                        double* rs, float* nrm, int* status) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= Ms) return;
   const double d = perm ? C[(int64_t)perm[i] * ldc + perm[i]] : *W.at(i, i);
   if (!(d > 0.0 && isfinite(d))) atomicExch(status, 1);
   rs[i] = 1.0 / sqrt(d);
+  nrm[i] = 0.0f;
 }
 
 // the selected rows, reordered and scaled, as integers; row Ms: D' (FP64)
@@ -246,6 +253,7 @@ struct FxPanel {
   int kb, kblk, nkb;     // columns; first K block of the panel in the buffer; its K blocks per row block
   uint8_t* dig;
   double *y, *ld, *ld_prev;  // solved data vector; this and the previous panel's diagonal factor (64 x 64)
+  float* nrm;                // squared norm of every row's factor entries so far
   int* status;
   int wide;  // the matrix is 16-byte aligned
 };
@@ -429,6 +437,18 @@ __global__ void __maxnreg__(104) k_fx_panel(FxPanel P) {
         P.ld[e] = i == l ? 1.0 / fx_rpivot(rinv[i], rsh[i]) : (double)fx_join(*(const int2*)&L[i][l]) * FX_Q57;
     }
     if (tid < kb) P.y[k0 + tid] = ysh[tid];
+    {
+      // the diagonal block's rows (the others: below), four threads each, without the pivot
+      const int i = tid >> 2;
+      float n2 = 0.0f;
+      for (int l = tid & 3; l < i; l += 4) {
+        const float f = __int2float_rn(((const int2*)&L[i][l])->x);
+        n2 = fmaf(f, f, n2);
+      }
+      n2 += __shfl_xor_sync(0xffffffffu, n2, 1);
+      n2 += __shfl_xor_sync(0xffffffffu, n2, 2);
+      if (i < kb && !(P.nrm[k0 + i] + n2 * 0x1p-62f <= FX_NORM)) atomicExch(P.status, 1);
+    }
     if (k0 > 0) fx_store_diag(W, k0 - FX_NB, FX_NB, P.ld_prev);
     return;
   }
@@ -437,9 +457,13 @@ __global__ void __maxnreg__(104) k_fx_panel(FxPanel P) {
   const int64_t row = r0 + rl;
   long long X[8];
   double xd[8], dot = 0.0;
+  float n2 = 0.0f;
 #pragma unroll
   for (int p = 0; p < 8; ++p) {
-    const long long v = fx_join(*(const int2*)&L[FX_NB + rl][8 * q + p]);
+    const int2 l = *(const int2*)&L[FX_NB + rl][8 * q + p];
+    const long long v = fx_join(l);
+    const float f = __int2float_rn(l.x);  // (units of 2^-31)
+    n2 = fmaf(f, f, n2);
     X[p] = (v + 2) >> 2;  // to units of 2^-55
     xd[p] = fx_double(v);
     dot = fma(xd[p], ysh[8 * q + p], dot);
@@ -447,7 +471,10 @@ __global__ void __maxnreg__(104) k_fx_panel(FxPanel P) {
   uint4 d[SL_S];
   sl_digits8(X, d);
 #pragma unroll
-  for (int o = 1; o < 8; o <<= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+  for (int o = 1; o < 8; o <<= 1) {
+    dot += __shfl_xor_sync(0xffffffffu, dot, o);
+    n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+  }
   if (rl < nr) {
     uint8_t* o = P.dig + ((size_t)((row >> 7) - P.rb0) * P.nkb + P.kblk + (q >> 2)) * SL_BLOCK +
                  (size_t)(row & 127) * (SL_BK * 2) + (q & 3) * 16;
@@ -458,7 +485,12 @@ __global__ void __maxnreg__(104) k_fx_panel(FxPanel P) {
     for (int p = 0; p < 8; p += 2)
       fx_st2(rowp + p, (unsigned long long)__double_as_longlong(xd[p]),
              (unsigned long long)__double_as_longlong(xd[p + 1]), P.wide);
-    if (q == 0) *W.at(P.Ms, row) -= dot;
+    if (q == 0) {
+      *W.at(P.Ms, row) -= dot;
+      const float t = P.nrm[row] + n2 * 0x1p-62f;
+      P.nrm[row] = t;
+      if (!(t <= FX_NORM)) atomicExch(P.status, 1);
+    }
   }
 }
 
@@ -605,10 +637,11 @@ int wl_num_sms() {
 }
 
 // scratch of a factorisation of n rows with super-panels of w panels: two digit
-// buffers, the diagonal factors of two panels, the solved data vector, the scaling
+// buffers, the diagonal factors of two panels, the solved data vector, the scaling, the rows'
+// norms
 size_t wl_fx_bytes(int64_t n, int w) {
   const size_t dig = (size_t)((n + SL_BM - 1) / SL_BM) * (size_t)(2 * w) * SL_BLOCK;
-  return 2 * dig + 2 * FX_NB * FX_NB * 8 + 16 * (size_t)((n + 1) / 2 * 2);
+  return 2 * dig + 2 * FX_NB * FX_NB * 8 + 16 * (size_t)((n + 1) / 2 * 2) + 4 * (size_t)((n + 1) / 2 * 2);
 }
 
 // The scratch, grown on demand: super-panels of four panels (eight for matrices whose
@@ -727,9 +760,10 @@ int wl_fx_factor(cov_handle* h, OutMap W, int64_t Ms, const int* perm, const dou
   double* ld = fx_tail_mem(h, Ms, w);
   double* y = ld + 2 * FX_NB * FX_NB;
   double* rs = y + (Ms + 1) / 2 * 2;
+  float* nrm = (float*)(rs + (Ms + 1) / 2 * 2);
   int* st = h->piv_status;
   int tk = wl_stage_begin(h, ST_SNR_PACK, s);
-  k_fx_rs<<<(unsigned)((Ms + 255) / 256), 256, 0, s>>>(Ms, perm, C, ldc, W, rs, st);
+  k_fx_rs<<<(unsigned)((Ms + 255) / 256), 256, 0, s>>>(Ms, perm, C, ldc, W, rs, nrm, st);
   if (perm) {
     k_fx_pack<<<dim3((unsigned)(Ms + 1), (unsigned)((Ms + 1023) / 1024)), 256, 0, s>>>(Ms, perm, C, ldc, D, rs, W.C, W.ldc,
                                                                                      st);
@@ -754,7 +788,7 @@ int wl_fx_factor(cov_handle* h, OutMap W, int64_t Ms, const int* perm, const dou
       const int64_t k0 = S0 + (int64_t)p * FX_NB;
       const int slot = (int)((k0 / FX_NB) & 1);
       FxPanel a{W, k0, Ms, S0 / SL_BM, (int)std::min<int64_t>(FX_NB, Ms - k0), 2 * p, nkb, fx_dig(h, Ms, w, b), y,
-                ld + slot * FX_NB * FX_NB, ld + (slot ^ 1) * FX_NB * FX_NB, st, fx_wide(W)};
+                ld + slot * FX_NB * FX_NB, ld + (slot ^ 1) * FX_NB * FX_NB, nrm, st, fx_wide(W)};
       const int64_t groups = std::max<int64_t>(0, (Ms - k0 - FX_NB + FX_RB - 1) / FX_RB);
       k_fx_panel<<<(unsigned)(groups + 1), FX_THREADS, FX_PSMEM, st_>>>(a);
       WL_LAUNCH(h, "k_fx_panel");
