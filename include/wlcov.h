@@ -247,8 +247,9 @@ int cov_assemble_band(cov_handle* h, int64_t row0, int64_t nrows, double* d_C, i
  * the lower-packed 256 x 256 tiles of rows 0..M, i.e. the tiles of M + 1 rows
  * ((t (t + 1) / 2) * 65536 doubles, t = M / 256 + 1), as written by
  * cov_assemble_band(h, 0, M, d_Ct, 0, COV_LAYOUT_TILES, ...).  d_Ct is
- * overwritten: Jacobi scaling, D' = d^-1/2 D (d_D: device, M) as row M, and
- * the same blocked FP64-accurate Cholesky as cov_snr; h_snr (host, n_ell)
+ * overwritten: the scaled matrix in fixed point, the scaled data vector (d_D:
+ * device, M) as row M, and the same blocked Cholesky as cov_snr, which leaves
+ * its FP64 factor; h_snr (host, n_ell)
  * receives S/N for ell_max = bin 0 .. n_ell - 1 of the handle's rows (P, B or
  * joint by the handle's row set).  COV_ERR_NOT_PD / COV_ERR_TIMEOUT as for
  * cov_snr; COV_ERR_INVALID for a handle not in cumulative order. */
@@ -256,8 +257,9 @@ int cov_snr_tiles(cov_handle* h, double* d_Ct, const double* d_D, double* h_snr,
 
 /* Cumulative signal-to-noise (Eqs. SNprim, eq:SN): h_snr[c] (host, n_ell
  * values) = sqrt(D^T C^-1 D) over the selected entries whose largest ell bin
- * is <= c, via a Jacobi-scaled FP64 Cholesky of a workspace copy (d_C is not
- * modified).  Returns COV_ERR_NOT_PD on a non-positive pivot.  Synchronises
+ * is <= c, via a Cholesky in 64-bit fixed point of a workspace copy, scaled to a
+ * diagonal of 1 (FP64 accuracy: entries to 2^-62, updates to 2^-53 of the
+ * diagonal; d_C is not modified).  Returns COV_ERR_NOT_PD on a non-positive pivot.  Synchronises
  * the stream. */
 int cov_snr(cov_handle* h, const double* d_C, int64_t ldc, const double* d_D, int which,
             double* h_snr, void* stream);
@@ -301,7 +303,7 @@ const char* cov_stage_name(int stage);
  * must never stall on an allocation.  The paper has no counterpart; this is a
  * deployment variant of cov_snr.
  *
- * It runs the same Jacobi-scaled FP64 Cholesky as cov_snr on d_C (device,
+ * It runs a Jacobi-scaled blocked FP64 Cholesky on d_C (device,
  * M x M lower triangle, row-major, leading dimension ldc >= M) and d_D
  * (device, M values), both already in cumulative order, and writes
  * d_snr[c] = sqrt(D^T C^-1 D) over the first prefix[c] entries, for

@@ -1,8 +1,8 @@
 // Cumulative signal-to-noise (paper Sec. 5, Eqs. SNprim and eq:SN).
 //
 // The selected entries (P, B or the joint vector) are reordered by their
-// largest ell bin (stable), Jacobi-scaled, C' = d^-1/2 C d^-1/2 and
-// D' = d^-1/2 D, and factorised in 64-bit fixed point (chol_fx.cu), which
+// largest ell bin (stable), scaled to a diagonal of 1, C' = S C S and D' = S D,
+// and factorised in 64-bit fixed point (chol_fx.cu), which
 // carries the data row along as y = L^-1 D'.  Because the leading principal
 // block of a Cholesky factor is the factor of the leading principal block,
 // (S/N)^2 for every cumulative ell_max is a prefix sum of y^2 over the

@@ -1,11 +1,14 @@
-// Blocked Cholesky of the unit-diagonal covariance in 64-bit fixed point (the S/N
-// solve of the paper's Sec. 5, Eqs. SNprim and eq:SN, and the factor of the PCA).
+// Blocked Cholesky of the scaled covariance in 64-bit fixed point (the S/N solve of the
+// paper's Sec. 5, Eqs. SNprim and eq:SN, and the factor of the PCA).
 //
-// After the Jacobi scaling C' = d^-1/2 C d^-1/2 every entry of the matrix, of each
-// Schur complement and of the factor is at most 1 in magnitude, and so is the 2-norm of
-// every factor row.  So the working matrix is held as integers in units of 2^-62: its
-// resolution is 2^-62 of the unit diagonal, where an FP64 entry near 1 has 2^-53, and
-// the elimination runs on the integer units.  A dependent FP64 operation takes 64
+// The rows and columns are scaled, C' = S C S, with scales of 24 bits close to C_ii^-1/2 and
+// the entries' products formed exactly: which scale is taken matters little, that it is the
+// same for every entry does (with FP64 products all of the S/N's error, 1.4e-14 at M = 632,
+// came from their roundings).  Every entry of the matrix, of each Schur complement and of the
+// factor is then below 1 in magnitude, and so is the 2-norm of every factor row.  So the
+// working matrix is held as integers in units of 2^-62: its resolution is 2^-62 of the
+// diagonal, where an FP64 entry near 1 has 2^-53, and the elimination runs on the integer
+// units.  A dependent FP64 operation takes 64
 // cycles on this part and an SM completes two per clock; a 64 x 64 -> 64-bit product is
 // a few 4-cycle multiply-adds.
 //
@@ -30,13 +33,16 @@
 // FP64 diagonal blocks and panel solves: the joint S/N of M = 6375 14.4 -> 7.9 ms, of
 // M = 818 1.28 -> 0.78 ms, the one in place at M = 24400 268 -> 158 ms.
 //
-// The integers are modulo 2^64, four times the unit diagonal.  In a positive definite matrix
+// The integers are modulo 2^64, i.e. modulo 4.  In a positive definite matrix
 // nothing leaves [-1, 1]; in another one a row wraps only after its factor entries' squares
 // have added up to more than its diagonal entry, so the panel kernel keeps that sum of every
 // row (FP32) and raises the pivot status beyond FX_NORM.
 //
-// Error: entries 2^-63 by rounding, updates 2^-56 per digit row against the unit
-// diagonal, i.e. below that of an FP64 factorisation (2^-53 per operation).
+// Error: entries 2^-62, factor entries 2^-58 inside a panel, updates 2^-56 per
+// digit row and 2^-53 per product, against the diagonal, i.e. below that of an FP64
+// factorisation (2^-53 per operation).  S/N against 80-bit factorisations of 24 matrices of 144
+// to 818 rows: the survey's 2e-16 .. 2.5e-15 (FP64 panels with slices of 2^-48: 9e-16 .. 1.7e-14),
+// Wishart matrices with pivots down to 5e-4 2e-13 .. 2e-11 (3e-11 .. 2e-9).
 #include <algorithm>
 
 #include "digits.cuh"
@@ -47,32 +53,31 @@
 // eight; no difference at 6375, where the scratch is then smaller)
 #define FX_WIDE 12288
 #define FX_ONE (1ll << 62)
-#define FX_NORM 1.0625f  // (at most 1 up to the FP32 sums' rounding, ~2e-4 at 2800 panels)
+#define FX_NORM 1.0625f  // (below 1 but for the FP32 sums' rounding, ~2e-4 at 2800 panels)
 
-// RN(x 2^62) for |x| <= 1 (2^-30 beyond counts as rounding); anything else, NaN
-// included, cannot be an entry of a scaled positive definite matrix: status
-__device__ __forceinline__ long long fx_fixed(double x, int* status) {
-  const double ax = fabs(x);
-  if (!(ax < 1.0)) {
-    if (!(ax <= 1.0 + 9.3e-10)) {
-      atomicExch(status, 1);
-      return 0;
-    }
-    return x < 0.0 ? -FX_ONE : FX_ONE;
+// RN(c s t 2^62) for |c s t| < 1, s and t scales of 24 bits (variance_scale): the 101-bit
+// product of the significands, of which 61 bits and more are kept before the rounding.
+// Anything else, NaN included, cannot be an entry of a scaled positive definite matrix: status
+__device__ __forceinline__ long long fx_fixed(double c, double s, double t, int* status) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(c);
+  const unsigned sh_ = (unsigned)__double2hiint(s), th = (unsigned)__double2hiint(t);
+  const int E = (int)((b >> 52) & 0x7FFu), Es = (int)(sh_ >> 20), Et = (int)(th >> 20);
+  if (E == 0x7FF) {
+    atomicExch(status, 1);
+    return 0;
   }
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const int E = (int)((b >> 52) & 0x7FFu);
+  if (E == 0 || Es == 0 || Et == 0) return 0;  // (a scale of 0 has raised the status)
   const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-  const int sh = 1013 - E;  // X = RN(m / 2^sh); sh >= -9
-  unsigned long long q;
-  if (sh <= 0) {
-    q = m << -sh;
-  } else if (sh >= 64) {
-    q = 0;
-  } else {
-    q = m >> sh;
-    const unsigned long long rem = m & ((1ull << sh) - 1), half = 1ull << (sh - 1);
-    q += (rem > half || (rem == half && (q & 1ull))) ? 1ull : 0ull;
+  const unsigned long long u = (unsigned long long)(((sh_ & 0xFFFFFu) | 0x100000u) << 3 | (unsigned)__double2loint(s) >> 29) *
+                               (((th & 0xFFFFFu) | 0x100000u) << 3 | (unsigned)__double2loint(t) >> 29);
+  const unsigned long long hi = __umul64hi(m << 11, u << 16);  // m u 2^-37: 61 to 64 bits
+  const int sh = 3068 - E - Es - Et;
+  unsigned long long q = 0;
+  if (sh > 0 && sh < 64) q = (hi >> sh) + ((hi >> (sh - 1)) & 1ull);
+  if (sh == 0) q = hi;
+  if (sh < 0 || q >= (unsigned long long)FX_ONE) {
+    atomicExch(status, 1);
+    return 0;
   }
   return (b >> 63) ? -(long long)q : (long long)q;
 }
@@ -95,15 +100,15 @@ __device__ __forceinline__ void fx_st2(double* p, unsigned long long a, unsigned
 }
 
 // ---------------------------------------------------------------- scaling
-// rs[i] = C_ii^-1/2 of the selected entries (perm null: row i of W, FP64); the scaled diagonal
-// is 1 by construction, so a variance that is no positive number is caught here
+// The scales rs[i] of the selected entries (perm null: row i of W, FP64).  A variance that is
+// no positive finite number is caught here.
 __global__ void k_fx_rs(int64_t Ms, const int* __restrict__ perm, const double* __restrict__ C, int64_t ldc, OutMap W,
                         double* rs, float* nrm, int* status) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= Ms) return;
   const double d = perm ? C[(int64_t)perm[i] * ldc + perm[i]] : *W.at(i, i);
   if (!(d > 0.0 && isfinite(d))) atomicExch(status, 1);
-  rs[i] = 1.0 / sqrt(d);
+  rs[i] = variance_scale(d);
   nrm[i] = 0.0f;
 }
 
@@ -125,7 +130,7 @@ __global__ void __launch_bounds__(256) k_fx_pack(int64_t Ms, const int* __restri
     if (j > i) break;
     const int64_t pj = perm[j];
     const int64_t hi = pi > pj ? pi : pj, lo = pi > pj ? pj : pi;
-    ((long long*)Wk)[i * ldw + j] = j == i ? FX_ONE - 1 : fx_fixed(C[hi * ldc + lo] * ri * rs[j], status);
+    ((long long*)Wk)[i * ldw + j] = fx_fixed(C[hi * ldc + lo], ri, rs[j], status);
   }
 }
 
@@ -148,7 +153,7 @@ __global__ void __launch_bounds__(256) k_fx_pack_tiles(int64_t M, OutMap W, cons
     if (r == M)
       *p = D[c] * rc;
     else
-      *(long long*)p = r == c ? FX_ONE - 1 : fx_fixed(*p * rc * rs[r], status);
+      *(long long*)p = fx_fixed(*p, rc, rs[r], status);
   }
 }
 

@@ -585,6 +585,14 @@ __device__ __forceinline__ double scaled_to_double_rn(long long a, int ex) {
   return __longlong_as_double((long long)(sign | (((unsigned long long)(e - 1) << 52) + r)));
 }
 
+// Scale of a covariance row for the fixed-point Cholesky: 1 / sqrt(d) of the variance d,
+// rounded down to 24 significant bits less one in the last, so that d s^2 is in (1 - 2^-21, 1)
+// and the product of two scales is exact; 0 for d that is no positive finite number
+__device__ __forceinline__ double variance_scale(double d) {
+  if (!(d > 0.0 && isfinite(d))) return 0.0;
+  return __longlong_as_double((__double_as_longlong(1.0 / sqrt(d)) & ~0x1FFFFFFFll) - 0x20000000ll);
+}
+
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

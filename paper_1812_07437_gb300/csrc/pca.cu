@@ -6,9 +6,9 @@
 // eigenvalue of a graded positive definite matrix, however small (the paper's
 // covariances span ~23 decades):
 //
-//  * the FP64-accurate Cholesky of the S/N (cov_snr) on the Jacobi-scaled matrix
-//    C' = d^-1/2 C d^-1/2, rows in order of descending C_aa, gives the factor L' and the
-//    solved data row y = L'^-1 d^-1/2 D = L^-1 D with L = d^1/2 L';
+//  * the FP64-accurate Cholesky of the S/N (cov_snr) on the scaled matrix C' = S C S
+//    (S ~ d^-1/2), rows in order of descending C_aa, gives the factor L' and the
+//    solved data row y = L'^-1 S D = L^-1 D with L = S^-1 L';
 //  * sweeps of plane rotations of column pairs make the columns of L orthogonal:
 //    L J = U diag(sigma), C = L L^T = U diag(sigma^2) U^T, so the eigenvalues are
 //    lambda_a = |l_a|^2.  With the large variances first, L's columns are graded and
@@ -33,7 +33,7 @@
 #define PCA_TOL 1e-15
 #define PCA_MAX_SWEEPS 60
 
-// Column j of L, contiguous: G[j][i] = sqrt(C_{p_i p_i}) x factor entry (i, j) (i >= j,
+// Column j of L, contiguous: G[j][i] = factor entry (i, j) / scale of row p_i (i >= j,
 // zero above), entry n the solved data row's y_j, the rest of the ld entries zero.
 // One 32 x 32 tile per CTA, transposed in shared memory.
 __global__ void __launch_bounds__(256) k_pca_build(int n, int ld, const double* __restrict__ W, int64_t ldw,
@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(256) k_pca_build(int n, int ld, const double* 
     double v = 0.0;
     if (i < n && j <= i) {
       const int64_t p = perm[i];
-      v = sqrt(C[p * ldc + p]) * W[(int64_t)i * ldw + j];
+      v = W[(int64_t)i * ldw + j] / variance_scale(C[p * ldc + p]);
     } else if (i == n && j < n) {
       v = W[(int64_t)n * ldw + j];
     }
