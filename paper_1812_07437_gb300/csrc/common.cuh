@@ -220,6 +220,7 @@ struct cov_handle {
   double *sl_w = nullptr, *sl_sr = nullptr;
   unsigned long long* sl_part = nullptr;  // exact partial sums of tiles shared by several CTAs, then their tickets
   int sl_rows = 0, sl_tri = 0;            // 0 undecided, 1 digits, -1 FP64 rows (k_gemm_lower)
+  bool sl_reserved = false;               // a server's reservation holds the digits
   double* work = nullptr;   // Cholesky workspace (M+1) rows
   int64_t work_n = 0;
   int64_t work_ld = 0;      // its row length (the last dense cov_snr)

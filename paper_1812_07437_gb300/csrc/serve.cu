@@ -167,7 +167,8 @@ static int run_request(cov_server* s, Rec& q, Resident* res, cudaStream_t stream
       q.err = cov_last_error(nullptr);
       return rc;
     }
-    // the FP64 form's digits only where the reservation holds them
+    // the FP64 form's digits where the reservation holds them, and only there
+    res->h->sl_reserved = q.digits;
     if (!q.digits) res->h->sl_rows = res->h->sl_tri = -1;
     const size_t M = (size_t)res->h->M;
     res->h->chol_scratch_cap = q.chol_cap;

@@ -779,8 +779,9 @@ int wl_sl_rows(cov_handle* h, bool tri, int nssc, cudaStream_t s) {
 // rows), and its buffers.  The digits take 14 bytes per entry where the FP64 rows of
 // k_gemm_lower take 8; where they do not fit (in hbm_budget, or the free memory, beside
 // all that the handle's other calls may still allocate) the FP64 rows and that kernel
-// serve the handle as before.  Decided
-// once per handle: a later call with more super-sample columns finds room for them.
+// serve the handle as before.  A served request's reservation was made with the digits in it,
+// so there they only have to fit.  Decided once per handle: a later call with more
+// super-sample columns finds room for them.
 int wl_sl_alloc(cov_handle* h, bool tri, bool* use, cudaStream_t s) {
   int& state = tri ? h->sl_tri : h->sl_rows;
   if (state) {
@@ -810,6 +811,7 @@ int wl_sl_alloc(cov_handle* h, bool tri, bool* use, cudaStream_t s) {
   WL_CHECK(h, cudaMemGetInfo(&fr, &tot));
   const size_t late = wl_late_bytes(h);
   bool ok = need <= fr / 4 * 3 && need + late <= fr && !(h->budget && h->allocated + need + late > h->budget);
+  if (h->sl_reserved) ok = need <= fr;  // (what the request allocates besides is in the same reservation)
   const bool had_trd = h->trd != nullptr;
   std::vector<void**> got;
   for (auto& a : al) {
