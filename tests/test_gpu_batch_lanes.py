@@ -43,3 +43,26 @@ def test_batch_equals_separate_calls(nt, nl, rows, budget):
                 assert np.array_equal(ref, got[k][w], equal_nan=True), (k, w)
     assert np.array_equal(got[0], again[0], equal_nan=True)
     h.close()
+
+
+# rows of all cosmologies from which the second workspace is taken, and the largest matrix for it (csrc/batch.cu)
+LANE_MIN_ROWS, LANE_MAX_ROWS = 2048, 8192
+
+
+@pytest.mark.parametrize("nt,nl,precision", [(3, 9, N.COV_FP64), (4, 9, N.COV_SPLIT_BF16)])
+def test_a_failed_factorisation_beside_another(nt, nl, precision):
+    """Without the terms that give power spectra a variance every factorisation of the step fails; the handle then gives
+    what it gave before, bit for bit."""
+    from paper_1812_07437_gb300.handle import Handle
+    wl = _wl(nt, nl)
+    cosmos = [dict(wl["cosmology"], sigma8=wl["cosmology"]["sigma8"] * f) for f in (1.0, 1.02, 0.97)]
+    h = Handle(wl)
+    assert (h.M - h.n_P) * len(cosmos) >= LANE_MIN_ROWS and h.M - h.n_P <= LANE_MAX_ROWS
+    ref, D, _ = h.batch_snr(cosmos, precision=precision, with_D=True)
+    for terms in (N.COV_TERM_PB, N.COV_TERM_BBPT | N.COV_TERM_PB):
+        with pytest.raises(N.CovError) as e:
+            h.batch_snr(cosmos, terms=terms, precision=precision)
+        assert e.value.code == N.COV_ERR_NOT_PD
+    got, D2, _ = h.batch_snr(cosmos, precision=precision, with_D=True)
+    assert np.array_equal(ref, got, equal_nan=True) and np.array_equal(D, D2)
+    h.close()
