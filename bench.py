@@ -352,12 +352,14 @@ def launches_per_step(which_sizes, n_tri, split, packed=False, M=0):
         # trispectrum table (rows_prep, pair signatures, BF16 rows, contraction) + factor rows (rows_prep,
         # signatures, BF16 rows) + inverse counts; then the contraction, the per-element products and the
         # Gaussian diagonal blocks, once or (large packed bands) once per sub-band of at least 64 waves of tiles
-        tb = (M + 255) // 256
-        n_sub = max(1, min(8, tb, int(0.5 * tb * (tb + 1) / 152 / 64))) if packed else 1
+        import torch
+        tb, sms = (M + 255) // 256, torch.cuda.get_device_properties(0).multi_processor_count
+        n_sub = max(1, min(8, tb, int(0.5 * tb * (tb + 1) / sms / 64))) if packed else 1
         assemble = 4 + 3 + 1 + 3 * n_sub
     else:
-        # trispectrum and factor rows (norms, digits, contraction each), inverse counts, products, Gaussian blocks
-        assemble = 3 + 3 + 1 + 1 + 1
+        # trispectrum and factor rows (rows_prep, weights, digits, exponents, contraction each), inverse counts,
+        # products, Gaussian blocks
+        assemble = 5 + 5 + 1 + 1 + 1
     snr = 0
     for ms in which_sizes:
         nb, w = (ms + 63) // 64, 8 if ms >= 12288 else 4

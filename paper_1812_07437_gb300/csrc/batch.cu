@@ -38,8 +38,7 @@ struct DevBuf {
 
 // A second set of what a factorisation works in: the P and B factorisations of a
 // step run beside the joint one.  Each is a chain of panels that leaves most of
-// the device idle: the three of M = 3064 take
-// 5.6 ms in turn and 3.1 ms so.  For the
+// the device idle: the three of M = 3064 take 5.6 ms in turn and 3.1 ms so.  For the
 // call only: it is given back when the call returns.
 #define LANE_MIN_ROWS 2048  // rows of all cosmologies: ~0.7 us saved for each, ~0.4 ms to set up
 #define LANE_MAX_ROWS 8192  // beyond, the updates fill the device (and the copy is > 0.5 GB)
@@ -58,8 +57,8 @@ struct Lane {
   }
 };
 
-// Not with a memory budget, for large matrices, or
-// when anything fails: the factorisations then run in turn.
+// Not with a memory budget, for large matrices, or when anything fails: the
+// factorisations then run in turn.
 void make_lane(cov_handle* h, int n, Lane* l) {
   const int64_t Ms = std::max(h->sel[COV_WHICH_P].Ms, h->sel[COV_WHICH_B].Ms);
   if (h->budget || h->chol_scratch_cap || Ms * n < LANE_MIN_ROWS || Ms > LANE_MAX_ROWS) return;

@@ -26,7 +26,7 @@
 #define WL_DUFFY_C (-1.01)
 #define WL_DUFFY_MPIVOT 2.0e12
 #define WL_DELTA_VIR 200.0
-#define WL_N_GL_CHI 64     // nodes of the chi(z) rule on [0, z]
+#define WL_N_GL_CHI 64     // nodes per piece of the source-redshift rules (the bins' norms, W_i)
 #define WL_N_ZS 64         // nodes per source-redshift piece of W_i
 #define WL_N_RK4 1024      // RK4 steps of the growth ODE
 #define WL_A_INIT 1.0e-3

@@ -71,9 +71,9 @@ __global__ void __launch_bounds__(HI_THREADS)
                const int32_t* __restrict__ tris, const double* __restrict__ m, const double* __restrict__ om,
                const double* __restrict__ f, const double* __restrict__ b1, const double* __restrict__ b2,
                const double* __restrict__ U, double* __restrict__ out) {
-  extern __shared__ double hs[];  // U, g2 b1 U, g2 b2 U, g3 U, g3 b1 U: [5][nl][HI_Q + 1], then six weights
+  extern __shared__ double hs[];  // U, g2 b1 U, g2 b2 U, g3 U, g3 b1 U: [5][nl][HI_Q + 1], then three weights
   const int n = blockIdx.x, LD = HI_Q + 1, S = nl * LD;
-  double* wt = hs + 5 * S;  // g1, g1 b1, g1 b2, g2 (per q)
+  double* wt = hs + 5 * S;  // g1 b1, g1 b2, g2 (per q)
   const double irho = 1.0 / (WL_RHO_CRIT0 * cosmo_p->Om);
   const int npair = nl * (nl + 1) / 2, nitem = nl + npair + ntri;
   const int it = blockIdx.y * HI_THREADS + threadIdx.x;

@@ -569,7 +569,7 @@ __device__ __forceinline__ bool sl_drain_aligned(unsigned long long (&acc)[SL_NG
 }
 
 struct SlArgs {
-  int64_t rows, row1, t0, t1;
+  int64_t row1, t0, t1;
   int nk, ns;                 // K blocks; CTAs that share a tile's K range
   const int* rexp;
   SlExp x;
@@ -874,7 +874,7 @@ int wl_sl_syrk(cov_handle* h, bool tri, int nssc, OutMap out, int64_t row1, cuda
       }
     }
   }
-  SlArgs a{rows, row1, t0, t1, (int)nk, ns, tri ? h->Texp : h->Aexp, x, out, h->tc_status,
+  SlArgs a{row1, t0, t1, (int)nk, ns, tri ? h->Texp : h->Aexp, x, out, h->tc_status,
            h->sl_report, h->sl_part, nullptr};
   a.ticket = (int*)(h->sl_part + (size_t)SL_SPLIT_TILES * SL_BM * SL_BM);
   if (ns > 1) {

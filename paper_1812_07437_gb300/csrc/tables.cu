@@ -396,7 +396,7 @@ struct NodeArgs {
   const cov_cosmology* cosmo;
   cov_bins b;
   int nchi, nsrc;
-  double zmax, ymax, theta;
+  double ymax, theta;
   const double *glcx, *glcw, *zint, *part, *kn, *kwt, *kws, *pk, *mb, *zsrc;
   double *scal, *chi, *wchi, *z, *Draw, *cz, *sig0, *dlns, *sigF, *rvir, *sigw2, *chis;
   double* ksum;
@@ -531,8 +531,8 @@ struct HaloArgs {
   cov_bins b;
   cov_nz nz;
   int nchi, nc, nl;
-  double zmax, ymax, st_amp;
-  const double *scal, *chi, *z, *Draw, *mb, *omb, *sig0, *dlns, *sigF, *zedges, *norms, *zsrc, *gsel, *chis;
+  double ymax, st_amp;
+  const double *scal, *chi, *z, *Draw, *mb, *omb, *sig0, *dlns, *sigF, *zedges, *norms, *gsel, *chis;
   const double *zint, *gx, *gw, *ell;
   double *D, *f, *b1, *b2, *W, *sigw2, *ac, *Pl, *dPl, *Psh;
 };
@@ -783,15 +783,15 @@ int wl_tables(cov_handle* h, cudaStream_t s) {
   const double ymax = log1p(nz.zmax);
   k_prep<<<WL_N_ZI + WL_N_K / WL_KT_THREADS, WL_KT_THREADS, 0, s>>>(c, ymax, h->chebm, h->knode, h->kw8, h->zint, h->pk,
                                                                    h->amp_part);
-  NodeArgs na{c,       b,       h->nchi,  nsrc,    nz.zmax, ymax,    h->theta, h->glcx, h->glcw, h->zint, h->amp_part,
-              h->knode, h->kwt, h->kws,   h->pk,   h->mb,   h->zsrc, h->scal,  h->chi,  h->wchi, h->z,    h->Draw,
-              h->cz,   h->sig0, h->dlns,  h->sigF, h->rvir, h->sigw2, h->chis, h->ksum, h->kticket};
+  NodeArgs na{c,       b,       h->nchi,  nsrc,    ymax,     h->theta, h->glcx, h->glcw, h->zint, h->amp_part,
+              h->knode, h->kwt, h->kws,   h->pk,   h->mb,    h->zsrc,  h->scal, h->chi,  h->wchi, h->z,    h->Draw,
+              h->cz,   h->sig0, h->dlns,  h->sigF, h->rvir,  h->sigw2, h->chis, h->ksum, h->kticket};
   k_nodes<<<h->nchi + 1 + WL_KSPLIT * (h->nmb + h->nchi) + (nsrc + GR_THREADS - 1) / GR_THREADS, GR_THREADS, 0, s>>>(na);
   const double sta =
       1.0 / (1.0 + pow(2.0, -WL_ST_P) * tgamma(0.5 - WL_ST_P) / sqrt(WL_PI));  // Sheth-Tormen normalisation
-  HaloArgs ha{c,       b,        nz,       h->nchi,  h->nc,   h->nl,   nz.zmax, ymax,    sta,     h->scal,
+  HaloArgs ha{c,       b,        nz,       h->nchi,  h->nc,   h->nl,   ymax,    sta,     h->scal,
               h->chi,  h->z,     h->Draw,  h->mb,    h->omb,  h->sig0, h->dlns, h->sigF, h->zedges, h->norms,
-              h->zsrc, h->gsel,  h->chis,  h->zint,  h->gl64x, h->gl64w, h->ell_d, h->D,  h->f,    h->b1,
+              h->gsel, h->chis,  h->zint,  h->gl64x, h->gl64w, h->ell_d, h->D,  h->f,    h->b1,
               h->b2,   h->W,     h->sigw2, h->ac,    h->Pl,   h->dPl,  h->Psh};
   const int npl = (h->nl * h->nchi * 8 + GR_THREADS - 1) / GR_THREADS;
   k_halo<<<(b.conc_model == COV_CONC_BULLOCK ? h->nmb : 0) + 2 * h->nchi + npl, GR_THREADS, 0, s>>>(ha);
