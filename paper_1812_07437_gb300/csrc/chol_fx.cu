@@ -286,9 +286,11 @@ __device__ __forceinline__ void fx_store_diag(const OutMap& W, int64_t k0, int k
 // diagonal factor and y) and takes eight columns at a time, one block barrier each:
 //  * warps 0-3 subtract the products of the eight columns before and factorise the eight
 //    columns of every remaining row, one row per lane in registers, each warp with its
-//    own copy of the 8 x 8 block in lanes 0-7: no barrier inside.  The pivot's chain (the
-//    reciprocal square root, one scaled entry, one shuffle, one product) is what bounds
-//    the panel;
+//    own copy of the 8 x 8 block in lanes 0-7: no barrier inside.  A warp may come to its
+//    copy after warp 0 has finished the block (other kernels' CTAs on the SM), so the
+//    factored entries inside an 8 x 8 block go to their mirror places above the diagonal,
+//    which nobody reads in these eight columns.  The pivot's chain (the reciprocal square
+//    root, one scaled entry, one shuffle, one product) is what bounds the panel;
 //  * meanwhile warps 4-6 subtract the products of all earlier columns from the next eight,
 //    and warp 7 advances y by the eight columns before.
 // One panel of M = 6375 (cold): 51 us for the FP64 diagonal block and 37 us for the FP64
@@ -329,6 +331,8 @@ __global__ void __maxnreg__(104) k_fx_panel(FxPanel P) {
     if (lane + 32 < kb) dv1 = *W.at(P.Ms, k0 + 32 + lane);
   }
   long long bad = 0;
+  // factored entry (i, l), l < i < 64: mirrored inside its 8 x 8 block
+  auto entry = [&](int i, int l) -> int2 { return *(const int2*)((i ^ l) < 8 ? &L[l][i] : &L[i][l]); };
   auto solve_y = [&](int c0) {  // warp 7: y of columns c0 .. c0 + 7, D' of the diagonal block's rows below
     double rd = 0.0;            // lane j < 8: 1 / L_jj
     if (lane < 8) rd = fx_rpivot(rinv[c0 + lane], rsh[c0 + lane]);
@@ -338,8 +342,8 @@ __global__ void __maxnreg__(104) k_fx_panel(FxPanel P) {
       const double yj = __shfl_sync(0xffffffffu, c < 32 ? dv0 : dv1, c & 31) * __shfl_sync(0xffffffffu, rd, j);
       if (lane == 0) ysh[c] = yj;
       const double ys = -yj * FX_Q57;
-      if (c < 31 && lane > c) dv0 = fma((double)fx_join(*(const int2*)&L[lane][c]), ys, dv0);
-      if (lane + 32 > c) dv1 = fma((double)fx_join(*(const int2*)&L[lane + 32][c]), ys, dv1);
+      if (c < 31 && lane > c) dv0 = fma((double)fx_join(entry(lane, c)), ys, dv0);
+      if (lane + 32 > c) dv1 = fma((double)fx_join(entry(lane + 32, c)), ys, dv1);
     }
   };
   __syncthreads();
@@ -350,10 +354,10 @@ __global__ void __maxnreg__(104) k_fx_panel(FxPanel P) {
       const int row = lane < 8 ? c0 + lane : c0 + 8 + warp * 24 + (lane - 8);
       const bool live = row < FX_ROWS;
       if (warp == 0 || c0 + 8 + warp * 24 < FX_ROWS) {
-        const int ro = live ? row : c0;
+        const int ro = live ? row : c0, last = lane < 8 ? lane : (live ? 7 : 0);
         long long a[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) a[k] = L[ro][c0 + k];
+        for (int k = 0; k < 8; ++k) a[k] = k <= last ? L[ro][c0 + k] : 0;
         if (c0 > 0) {  // minus the products of the eight columns before (the earlier ones: warps 4-6)
           FxAcc v[8];
 #pragma unroll
@@ -393,7 +397,11 @@ __global__ void __maxnreg__(104) k_fx_panel(FxPanel P) {
             if (k == j + 1) d = fx_sub(dn, y, y);
             a[k] = fx_sub(a[k], l, y);
           }
-          if (live && (lane >= 8 || (warp == 0 && lane > j))) *(int2*)&L[row][c0 + j] = l;
+          if (lane < 8) {
+            if (warp == 0 && lane > j) *(int2*)&L[c0 + j][row] = l;
+          } else if (live) {
+            *(int2*)&L[row][c0 + j] = l;
+          }
         }
       }
     } else if (warp < 7) {
@@ -439,7 +447,7 @@ __global__ void __maxnreg__(104) k_fx_panel(FxPanel P) {
     for (int e = tid; e < FX_NB * FX_NB; e += FX_THREADS) {
       const int i = e >> 6, l = e & 63;
       if (i < kb && l <= i)
-        P.ld[e] = i == l ? 1.0 / fx_rpivot(rinv[i], rsh[i]) : (double)fx_join(*(const int2*)&L[i][l]) * FX_Q57;
+        P.ld[e] = i == l ? 1.0 / fx_rpivot(rinv[i], rsh[i]) : (double)fx_join(entry(i, l)) * FX_Q57;
     }
     if (tid < kb) P.y[k0 + tid] = ysh[tid];
     {
@@ -447,7 +455,7 @@ __global__ void __maxnreg__(104) k_fx_panel(FxPanel P) {
       const int i = tid >> 2;
       float n2 = 0.0f;
       for (int l = tid & 3; l < i; l += 4) {
-        const float f = __int2float_rn(((const int2*)&L[i][l])->x);
+        const float f = __int2float_rn(entry(i, l).x);
         n2 = fmaf(f, f, n2);
       }
       n2 += __shfl_xor_sync(0xffffffffu, n2, 1);
