@@ -336,14 +336,19 @@ __global__ void __maxnreg__(104) k_fx_panel(FxPanel P) {
   auto solve_y = [&](int c0) {  // warp 7: y of columns c0 .. c0 + 7, D' of the diagonal block's rows below
     double rd = 0.0;            // lane j < 8: 1 / L_jj
     if (lane < 8) rd = fx_rpivot(rinv[c0 + lane], rsh[c0 + lane]);
+    // row lane (c0 < 32) or lane + 32: the columns c0 .. of the row, or of the block's mirror
+    const bool m0 = (lane ^ c0) < 8, m1 = ((lane + 32) ^ c0) < 8;
+    const long long *p0 = m0 ? &L[c0][lane] : &L[lane][c0], *p1 = m1 ? &L[c0][lane + 32] : &L[lane + 32][c0];
 #pragma unroll 1
     for (int j = 0; j < 8; ++j) {
       const int c = c0 + j;
       const double yj = __shfl_sync(0xffffffffu, c < 32 ? dv0 : dv1, c & 31) * __shfl_sync(0xffffffffu, rd, j);
       if (lane == 0) ysh[c] = yj;
       const double ys = -yj * FX_Q57;
-      if (c < 31 && lane > c) dv0 = fma((double)fx_join(entry(lane, c)), ys, dv0);
-      if (lane + 32 > c) dv1 = fma((double)fx_join(entry(lane + 32, c)), ys, dv1);
+      if (c < 31 && lane > c) dv0 = fma((double)fx_join(*(const int2*)p0), ys, dv0);
+      if (lane + 32 > c) dv1 = fma((double)fx_join(*(const int2*)p1), ys, dv1);
+      p0 += m0 ? FX_LD : 1;
+      p1 += m1 ? FX_LD : 1;
     }
   };
   __syncthreads();
@@ -371,6 +376,10 @@ __global__ void __maxnreg__(104) k_fx_panel(FxPanel P) {
 #pragma unroll
           for (int k = 0; k < 8; ++k) a[k] = v[k].value();
         }
+        // where this lane's factored entries go, and the step from one column to the next
+        int2* out = lane < 8 ? (int2*)&L[c0][row] : (int2*)&L[ro][c0];
+        const int step = lane < 8 ? FX_LD : 1;
+        const int upto = lane < 8 ? (warp == 0 ? lane : 0) : (live ? 8 : 0);  // columns below this one
         long long d = fx_bcast(a[0], 0);
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
@@ -397,11 +406,7 @@ __global__ void __maxnreg__(104) k_fx_panel(FxPanel P) {
             if (k == j + 1) d = fx_sub(dn, y, y);
             a[k] = fx_sub(a[k], l, y);
           }
-          if (lane < 8) {
-            if (warp == 0 && lane > j) *(int2*)&L[c0 + j][row] = l;
-          } else if (live) {
-            *(int2*)&L[row][c0 + j] = l;
-          }
+          if (j < upto) out[j * step] = l;
         }
       }
     } else if (warp < 7) {
