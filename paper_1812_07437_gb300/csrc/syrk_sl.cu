@@ -32,7 +32,7 @@
 // block).  K blocks that add nothing to a tile are not read (SlLive).  M = 6375, 400 K blocks:
 // contraction 7.1 ms where k_gemm_lower took 415 + 4.4 ms (1.2 TFLOP/s), trispectrum table
 // 37 -> 1.0 ms, rows 0.51 ms, whole FP64 assembly 464 -> 9.0 ms.  M = 818 (28 tiles in 5 parts
-// each): contraction 0.29 ms, assembly 27.1 -> 0.68 ms.  (With one exponent per row: 11.8 and
+// each): contraction 0.29 ms, assembly 27.1 -> 0.66 ms.  (With one exponent per row: 11.8 and
 // 0.63 ms.)
 #include "digits.cuh"
 
@@ -158,47 +158,62 @@ __host__ __device__ static inline SlExp sl_exp(uint8_t* dig, int64_t nb, int64_t
 }
 
 // The distances, and the row's largest exponent (0 for an empty row, SL_BAD for one that is
-// not finite).  One CTA per row block, a thread per row and every eighth group.
+// not finite).  One CTA per row block; a warp holds all 128 rows, four to a lane, of every 32nd
+// K block or group (bound by the latency of its passes: 16 us with a row to a thread).
 __global__ void __launch_bounds__(1024) k_sl_exp(SlExp x, int64_t rows, int* rexp) {
-  __shared__ int mx[8][SL_BM];
-  const int r = threadIdx.x & (SL_BM - 1), y = threadIdx.x >> 7;
+  __shared__ int4 mx[32][SL_BM / 4];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t rb = blockIdx.x;
-  const int16_t* e = x.e + (size_t)rb * x.nk * SL_BM + r;
-  int m = SL_EMPTY;
+  const short4* e = (const short4*)(x.e + (size_t)rb * x.nk * SL_BM) + lane;
+  int m[4] = {SL_EMPTY, SL_EMPTY, SL_EMPTY, SL_EMPTY};
 #pragma unroll 4
-  for (int k = y; k < x.nk; k += 8) m = max(m, (int)e[(size_t)k * SL_BM]);
-  mx[y][r] = m;
+  for (int k = warp; k < x.nk; k += 32) {
+    const short4 v = e[(size_t)k * (SL_BM / 4)];
+    m[0] = max(m[0], (int)v.x);
+    m[1] = max(m[1], (int)v.y);
+    m[2] = max(m[2], (int)v.z);
+    m[3] = max(m[3], (int)v.w);
+  }
+  mx[warp][lane] = make_int4(m[0], m[1], m[2], m[3]);
   __syncthreads();
+#pragma unroll 8
+  for (int i = 0; i < 32; ++i) {
+    const int4 v = mx[i][lane];
+    m[0] = max(m[0], v.x);
+    m[1] = max(m[1], v.y);
+    m[2] = max(m[2], v.z);
+    m[3] = max(m[3], v.w);
+  }
 #pragma unroll
-  for (int i = 0; i < 8; ++i) m = max(m, mx[i][r]);
-  if (m == SL_EMPTY) m = 0;
-  if (y == 0 && rb * SL_BM + r < rows) rexp[rb * SL_BM + r] = m;
-  uint8_t* d = x.d + (size_t)rb * x.nk * SL_BM + r;
+  for (int c = 0; c < 4; ++c) {
+    if (m[c] == SL_EMPTY) m[c] = 0;
+    const int64_t r = rb * SL_BM + 4 * lane + c;
+    if (warp == 0 && r < rows) rexp[r] = m[c];
+  }
+  uchar4* d = (uchar4*)(x.d + (size_t)rb * x.nk * SL_BM) + lane;
 #pragma unroll 2
-  for (int g = y; g < x.ng; g += 8) {
-    int lo = SL_NONE;
+  for (int g = warp; g < x.ng; g += 32) {
+    int lo[4] = {SL_NONE, SL_NONE, SL_NONE, SL_NONE};
 #pragma unroll
     for (int i = 0; i < SL_GB; ++i) {
       const int k = g * x.gb + i;
       if (i < x.gb && k < x.nk) {
-        const int below = m - (int)e[(size_t)k * SL_BM], v = below > SL_FAR ? SL_NONE : below;
-        d[(size_t)k * SL_BM] = (uint8_t)v;
-        lo = min(lo, v);
+        const short4 s = e[(size_t)k * (SL_BM / 4)];
+        const int at[4] = {s.x, s.y, s.z, s.w};
+        int v[4], least = SL_NONE;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          v[c] = m[c] - at[c] > SL_FAR ? SL_NONE : m[c] - at[c];
+          lo[c] = min(lo[c], v[c]);
+          least = min(least, v[c]);
+        }
+        d[(size_t)k * (SL_BM / 4)] = make_uchar4((uint8_t)v[0], (uint8_t)v[1], (uint8_t)v[2], (uint8_t)v[3]);
+        least = __reduce_min_sync(0xffffffffu, least);
+        if (lane == 0) x.bd[(size_t)rb * x.nk + k] = (uint8_t)least;
       }
     }
-    x.gd[((size_t)rb * x.ng + g) * SL_BM + r] = (uint16_t)lo;
-  }
-  __syncthreads();
-  for (int k = threadIdx.x; k < x.nk; k += 1024) {
-    const uint4* p = (const uint4*)(x.d + ((size_t)rb * x.nk + k) * SL_BM);
-    uint32_t lo = 0xFFFFFFFFu;
-#pragma unroll
-    for (int i = 0; i < SL_BM / 16; ++i) {
-      const uint4 w = p[i];
-      lo = __vminu4(__vminu4(lo, __vminu4(w.x, w.y)), __vminu4(w.z, w.w));
-    }
-    lo = __vminu4(lo, lo >> 16);
-    x.bd[(size_t)rb * x.nk + k] = (uint8_t)min(lo & 255u, (lo >> 8) & 255u);
+    *((ushort4*)(x.gd + ((size_t)rb * x.ng + g) * SL_BM) + lane) =
+        make_ushort4((uint16_t)lo[0], (uint16_t)lo[1], (uint16_t)lo[2], (uint16_t)lo[3]);
   }
 }
 
@@ -374,6 +389,7 @@ __device__ __forceinline__ int sl_bound(const uint16_t* gi, const uint16_t* gj, 
   for (int c0 = 0; c0 < x.ng; c0 += SL_CHUNK) {
     const int cn = min(SL_CHUNK, x.ng - c0);
     if (c0) asm volatile("bar.sync 1, 256;" ::: "memory");
+#pragma unroll 4
     for (int e = threadIdx.x & 255; e < cn * (SL_BM / 8); e += 256) {
       si[e] = __ldg((const uint4*)(gi + (size_t)c0 * SL_BM) + e);
       sj[e] = __ldg((const uint4*)(gj + (size_t)c0 * SL_BM) + e);
